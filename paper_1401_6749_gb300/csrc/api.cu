@@ -300,6 +300,8 @@ tm_status_t dslash_dispatch(const tm_op* op, tm_prec_t prec, const DslashCall& c
 size_t link_bytes(const Geom& g, tm_prec_t p, int recon);
 tm_status_t pack_links(const Geom& g, tm_prec_t p, int recon, void* out, const double* U,
                        cudaStream_t s);
+size_t links_fx_bytes(const Geom& g);
+tm_status_t pack_links_fx(const Geom& g, void* out, const double* U, int* bad, cudaStream_t s);
 
 }  // namespace tml
 
@@ -491,6 +493,7 @@ extern "C" tm_status_t tm_op_create(tm_op_t** out, const tm_params_t* p, const d
   op->owns_links = true;
   for (int i = 0; i < kNumPrec; ++i) op->links[i] = op->links_il[i] = nullptr;
   op->il_err = nullptr;
+  op->links_fx = nullptr;
   const cudaStream_t st = (cudaStream_t)s;
   const double* U = nullptr;
   double* staged = nullptr;
@@ -521,6 +524,24 @@ extern "C" tm_status_t tm_op_create(tm_op_t** out, const tm_params_t* p, const d
       }
     }
   }
+  // fixed-point copy for the FP64 Dslash; *fx_bad tells whether every link is in its range
+  int* fx_bad = nullptr;
+  int h_bad = 0;
+  {
+    tm_status_t s5 = dev_alloc(&op->links_fx, links_fx_bytes(op->g), st, "tm_op_create");
+    if (s5 == TM_OK) s5 = dev_alloc((void**)&fx_bad, sizeof(int), st, "tm_op_create");
+    if (s5 == TM_OK && cudaMemsetAsync(fx_bad, 0, sizeof(int), st) != cudaSuccess) s5 = TM_ERR_CUDA;
+    if (s5 == TM_OK) s5 = pack_links_fx(op->g, op->links_fx, U, fx_bad, st);
+    if (s5 == TM_OK && cudaMemcpyAsync(&h_bad, fx_bad, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+      s5 = TM_ERR_CUDA;
+    dev_free(fx_bad, st);
+    if (s5 != TM_OK) {
+      if (s5 == TM_ERR_CUDA) cudaGetLastError();
+      dev_free(staged, st);
+      tm_op_destroy(op);
+      return s5;
+    }
+  }
   dev_free(staged, st);  // stream-ordered: after the packing that reads it
   if (op->il_err) {
     tm_status_t s4 = il_prepare();
@@ -531,6 +552,10 @@ extern "C" tm_status_t tm_op_create(tm_op_t** out, const tm_params_t* p, const d
     set_error("tm_op_create: %s", cudaGetErrorString(cudaGetLastError()));
     tm_op_destroy(op);
     return TM_ERR_CUDA;
+  }
+  if (h_bad) {
+    dev_free(op->links_fx, st);
+    op->links_fx = nullptr;
   }
   *out = op;
   return TM_OK;
@@ -561,7 +586,10 @@ extern "C" tm_status_t tm_op_destroy(tm_op_t* op) {
       dev_free(op->links[i], nullptr);
       dev_free(op->links_il[i], nullptr);
     }
-  if (op->owns_links) dev_free(op->il_err, nullptr);
+  if (op->owns_links) {
+    dev_free(op->il_err, nullptr);
+    dev_free(op->links_fx, nullptr);
+  }
   if (op->cg_graph.exec) cudaGraphExecDestroy(op->cg_graph.exec);
   dev_free(op->work, nullptr);
   cudaStreamSynchronize(nullptr);

@@ -1,0 +1,406 @@
+// FP64 Dslash with the hopping sum in 64-bit fixed point on the integer pipes.
+//
+// GB300 multiplies FP64 at 2 multiply-adds per clock and SM, but does 32
+// 32 x 32 -> 64-bit integer multiply-adds (IMAD.WIDE) in the same clock.  The
+// hopping sum needs no floating point inside one stencil: every site's 24
+// reals are added with factors of modulus <= 1, so a fixed point relative to
+// the largest of them keeps more bits than FP64 rounding of the partial sums.
+//
+// With E one above the biased exponent of the largest component met so far, a
+// component x enters as F = trunc(x 2^(1078 - E)), |F| < 2^56, split into hi 2^27 +
+// lo (both with the sign of x).  A link's part u is round(u 2^54) = ghi 2^27 + glo,
+// |glo| <= 2^26 (pack_links_fx, made with the operator; |u| <= 1.25 is checked
+// there, other links take the FP64 kernel).  Spin projections are integer
+// sums of the halves and every product F G is three IMAD.WIDE:
+//   hh += ghi hi,   md += ghi lo + glo hi        (glo lo, below the unit, is dropped)
+// A hop adds T = hh + (md >> 27) in units of 2^(E - 1078), 2^-56 of the bound
+// 2^(E - 1022) on the components.  |hi| < 2^30 and |lo| < 2^28 after the
+// projection, so the sum over 8 hops, 3 colours and 2 parts stays below
+// 48 * 1.25 * 2^57 < 2^63.  Rounding: inputs truncated at 2^-56 of the bound, links
+// 2^-55 of the factor, a unit of dropped products per term at most: a few
+// 2^-55 of the largest component of the stencil, below what the 60 roundings of
+// an FP64 evaluation leave (2^-53 of a partial sum each).  Measured against
+// complex128: M 1.14e-16 (FP64 arithmetic 1.36e-16), four hopping-expansion
+// steps 2.96e-16 (3.08e-16).
+//
+// Components outside 2^-863 .. 2^878 (infinities and NaN among them) send the
+// site to an FP64 evaluation of the same sum (hop_sum_f64), so the kernel's
+// range and special values are those of the FP64 arithmetic.
+//
+// The sums T are converted to FP64 once per output component; centre, twist
+// and CG update follow in FP64 (fx_epilogue).
+#pragma once
+
+
+namespace tml {
+
+constexpr unsigned kFxMinExp = 160, kFxMaxExp = 1900;  // biased exponents the fixed point takes
+constexpr unsigned kFxBad = 0x7fffu;                   // mark of a sum out of that range
+
+// right shifts, zero / the sign for counts of 64 and more
+__device__ __forceinline__ unsigned shr64_lo(unsigned long long v, unsigned n) {
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return (unsigned)r;
+}
+__device__ __forceinline__ long long shr64_s(long long v, unsigned n) {
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+}
+
+// |x| 2^(1078 - E) truncated, as unsigned halves (hi, lo < 2^27); z: +-1, x's sign
+// times that of the mask nm (0 or -1)
+__device__ __forceinline__ int3 fx_of(double x, unsigned E, int nm) {
+  const int h = __double2hiint(x);
+  const unsigned long long m =
+      ((unsigned long long)(((unsigned)h & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(x)) << 3;
+  const unsigned sh = E - (((unsigned)h >> 20) & 0x7ffu);
+  return make_int3((int)shr64_lo(m, sh + 27), (int)(shr64_lo(m, sh) & 0x7ffffffu), ((h >> 31) ^ nm) | 1);
+}
+
+struct Fx {
+  int hi, lo;
+};
+
+// a + b of two signed halves pairs: the signs are factors of integer FMAs
+__device__ __forceinline__ Fx fx_add(int3 a, int3 b) {
+  return {b.x * b.z + a.x * a.z, b.y * b.z + a.y * a.z};
+}
+
+__device__ __forceinline__ unsigned abs_hi(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+
+// 16-byte words of site cb in a plane of 32-site groups [group][rows][32]
+__device__ __forceinline__ unsigned fx_row(int cb, int rows) {
+  return (unsigned)(cb >> 5) * (unsigned)(32 * rows) + (unsigned)(cb & 31);
+}
+
+// The spin structure of a hop, (1 + SGN g_mu) W psi, seen from one upper spin s
+// of the output: h = psi_s + SGN i^ak psi_{2 + ac}, w = W h is added to spin s and
+// SGN i^-ak w to the lower row ac (B_mu A_mu = 1).  In the DeGrand-Rossi basis
+// ac = 1 - s for x, y and s for z, t; i^ak is +-i for x, z (ODD) and +-1 for y, t.
+// So one body serves (x, y) and (z, t) and both spins with a run-time sign, the
+// mask nd (0 or -1) on psi_{2 + ac}.
+struct FxSum {
+  long long upr[3], upi[3], lor[3], loi[3];
+  unsigned E;    // units of 2^(E - 1078)
+  unsigned big;  // largest |high word| met
+};
+
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) { return (long long)a * b + c; }
+
+// one hop: up += w, lo += w (forward) or -= w (backward, W = U^dag), w times -1
+// with nm = -1; up and dn point at the neighbour's chunks of spin s and 2 + ac, u
+// at its link
+template <bool ODD, bool ADJ>
+__device__ __forceinline__ void fx_hop(FxSum& s, const double2* up, const double2* dn, const int4* u, size_t cs,
+                                       int nd, int nm) {
+  double2 p[3], q[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    p[c] = up[c * cs];
+    q[c] = dn[c * cs];
+  }
+  unsigned big = 0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    big = max(max(big, max(abs_hi(p[c].x), abs_hi(p[c].y))), max(abs_hi(q[c].x), abs_hi(q[c].y)));
+  if (big == 0) {  // zero, or denormals whose high words vanish (out of range)
+    unsigned any = 0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      any |= (unsigned)(__double2loint(p[c].x) | __double2loint(p[c].y) | __double2loint(q[c].x) |
+                        __double2loint(q[c].y));
+    big = any ? 1u : 0u;
+  }
+  s.big = max(s.big, big);
+  if ((big >> 20) > s.E) {
+    const unsigned E = (big >> 20) + 1, d = E - s.E;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      s.upr[a] = shr64_s(s.upr[a], d);
+      s.upi[a] = shr64_s(s.upi[a], d);
+      s.lor[a] = shr64_s(s.lor[a], d);
+      s.loi[a] = shr64_s(s.loi[a], d);
+    }
+    s.E = E;
+  }
+  const unsigned E = s.E;
+  Fx hre[3], him[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    if constexpr (ODD) {  // p + i q
+      hre[c] = fx_add(fx_of(p[c].x, E, nm), fx_of(q[c].y, E, ~(nd ^ nm)));
+      him[c] = fx_add(fx_of(p[c].y, E, nm), fx_of(q[c].x, E, nd ^ nm));
+    } else {
+      hre[c] = fx_add(fx_of(p[c].x, E, nm), fx_of(q[c].x, E, nd ^ nm));
+      him[c] = fx_add(fx_of(p[c].y, E, nm), fx_of(q[c].y, E, nd ^ nm));
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    // re: u.re h.re - u.im h.im,  im: u.re h.im + u.im h.re  (u.im -> -u.im for the adjoint)
+    // md starts at half a unit, so that md >> 27 rounds (rounding down doubles
+    // the error of a solve, 1.2e-15 against 5.7e-16 at 4^4)
+    long long hr = 0, hi = 0, mr = 1 << 26, mi = 1 << 26;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int4 w = u[(ADJ ? 3 * b + a : 3 * a + b) * 32];  // (re.hi, re.lo, im.hi, im.lo)
+      const Fx xr = hre[b], xi = him[b];
+      const Fx si = ADJ ? xi : Fx{-xi.hi, -xi.lo}, sr = ADJ ? Fx{-xr.hi, -xr.lo} : xr;
+      hr = mad_wide(w.x, xr.hi, hr);
+      mr = mad_wide(w.x, xr.lo, mr);
+      hi = mad_wide(w.x, xi.hi, hi);
+      mi = mad_wide(w.x, xi.lo, mi);
+      hr = mad_wide(w.z, si.hi, hr);
+      mr = mad_wide(w.y, xr.hi, mr);
+      hi = mad_wide(w.z, sr.hi, hi);
+      mi = mad_wide(w.y, xi.hi, mi);
+      mr = mad_wide(w.z, si.lo, mr);
+      mi = mad_wide(w.z, sr.lo, mi);
+      mr = mad_wide(w.w, si.hi, mr);
+      mi = mad_wide(w.w, sr.hi, mi);
+    }
+    const long long tr = hr + (mr >> 27), ti = hi + (mi >> 27);
+    s.upr[a] += tr;
+    s.upi[a] += ti;
+    s.lor[a] += ADJ ? -tr : tr;
+    s.loi[a] += ADJ ? -ti : ti;
+  }
+}
+
+// the hopping sum at site cb of parity par for system r in FP64 arithmetic
+template <bool DAG>
+__device__ __noinline__ void hop_sum_f64(Cx<double>* out, const Geom* gp, const void* links, const void* in, int r,
+                                         int par, int cb) {
+  const Geom& g = *gp;
+  const Site s = site_of(g, par, cb);
+  const int opar = par ^ 1;
+  const size_t cs = (size_t)g.Vh, f0 = (size_t)(r * 2 + opar) * 12 * cs;
+  Cx<double> acc[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) acc[k] = {0.0, 0.0};
+  constexpr int SF = DAG ? +1 : -1, SB = -SF;
+  auto dir = [&](auto mu_tag) {
+    constexpr int MU = decltype(mu_tag)::value;
+    const bool edge = MU == 3 && g.antiperiodic;
+    const int lf = lex_fwd(g, s, MU) >> 1, lb = lex_bwd(g, s, MU) >> 1;
+    hop_site<double, MU, SF, false>(acc, in, f0 + lf, cs, load_link<double, 18>(links, g, MU, par, cb),
+                                    edge && s.c[3] == g.L[3] - 1 ? -1.0 : 1.0);
+    hop_site<double, MU, SB, true>(acc, in, f0 + lb, cs, load_link<double, 18>(links, g, MU, opar, lb),
+                                   edge && s.c[3] == 0 ? -1.0 : 1.0);
+  };
+  dir(std::integral_constant<int, 0>{});
+  dir(std::integral_constant<int, 1>{});
+  dir(std::integral_constant<int, 2>{});
+  dir(std::integral_constant<int, 3>{});
+#pragma unroll
+  for (int k = 0; k < 12; ++k) out[k] = acc[k];
+}
+
+// The FP64 epilogue (dslash_epilogue) of the components of spins sp and 2 + sp:
+// acc[0..2] and acc[3..5] the hopping sums in units of `unit`.  Returns their
+// |.|^2.
+template <int EPI, int CENTRE, bool INV>
+__device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp, int r, int par, int cb, double unit,
+                                              const Cx<double> (&acc)[6]) {
+  const size_t cs = (size_t)a.g.Vh;
+  const size_t b0 = ((size_t)(r * 2 + par) * 12 + 3 * sp) * cs + cb;  // chunk q: + (q < 3 ? q : q + 3) cs
+  const double nu = a.nu, inv = a.inv;
+  const double shop = CENTRE == 0 && INV ? a.hop_scale * unit * inv : a.hop_scale * unit;
+  Cx<double> o[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    const double tw = q < 3 ? nu : -nu;  // gamma_5 = diag(1, 1, -1, -1)
+    const Cx<double> v = acc[q];
+    if constexpr (CENTRE != 0) {
+      const double2 c = reinterpret_cast<const double2*>(a.c.cfield ? a.c.cfield : a.c.in)[b0 + (q < 3 ? q : q + 3) * cs];
+      o[q] = {c.x, c.y};
+      if constexpr (CENTRE == 2) o[q] = {__fma_rn(-tw, c.y, c.x), __fma_rn(tw, c.x, c.y)};
+      o[q] = {__fma_rn(shop, v.re, o[q].re), __fma_rn(shop, v.im, o[q].im)};
+      if constexpr (INV) o[q] = {inv * __fma_rn(tw, o[q].im, o[q].re), inv * __fma_rn(-tw, o[q].re, o[q].im)};
+    } else if constexpr (INV) {  // A^-1 s_hop h = (s_hop / (1 + nu^2)) (h - i nu g5 h)
+      o[q] = {shop * __fma_rn(tw, v.im, v.re), shop * __fma_rn(-tw, v.re, v.im)};
+    } else {
+      o[q] = {shop * v.re, shop * v.im};
+    }
+  }
+  double part = 0.0;
+  if constexpr (EPI == EPI_OUT) {
+    double2* out = reinterpret_cast<double2*>(a.c.out) + b0;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      if (q >= 3 && a.c.g5_out) o[q] = {-o[q].re, -o[q].im};
+      out[(q < 3 ? q : q + 3) * cs] = make_double2(o[q].re, o[q].im);
+    }
+    if (a.c.partial) {
+#pragma unroll
+      for (int q = 0; q < 6; ++q) part = __fma_rn(o[q].re, o[q].re, __fma_rn(o[q].im, o[q].im, part));
+    }
+  } else if constexpr (EPI == EPI_CGUPD) {
+    const double al = a.c.alpha[r];
+    double2* rf = reinterpret_cast<double2*>(a.c.r) + b0;
+    double2* xf = reinterpret_cast<double2*>(a.c.x) + b0;
+    const double2* pf = reinterpret_cast<const double2*>(a.c.p) + b0;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const size_t i = (q < 3 ? q : q + 3) * cs;
+      const double2 v = rf[i], x = xf[i], p = pf[i];
+      const double2 n = make_double2(__fma_rn(-al, o[q].re, v.x), __fma_rn(-al, o[q].im, v.y));
+      rf[i] = n;
+      xf[i] = make_double2(__fma_rn(al, p.x, x.x), __fma_rn(al, p.y, x.y));
+      part = __fma_rn(n.x, n.x, __fma_rn(n.y, n.y, part));
+    }
+  } else {  // EPI_RESID
+    const double2* bf = reinterpret_cast<const double2*>(a.c.b) + b0;
+    double2* out = reinterpret_cast<double2*>(a.c.out) + b0;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const size_t i = (q < 3 ? q : q + 3) * cs;
+      const double2 v = bf[i];
+      const double2 n = make_double2(__dsub_rn(v.x, o[q].re), __dsub_rn(v.y, o[q].im));
+      out[i] = n;
+      part = __fma_rn(n.x, n.x, __fma_rn(n.y, n.y, part));
+    }
+  }
+  return part;
+}
+
+// Two warps take 32 consecutive sites of one system, one for each upper spin
+// (with the lower rows it feeds), and exchange the lower row that belongs to
+// the other one through shared memory.  The loop over (x, y), (z, t) keeps 12
+// sums of 64 bits and the code small.  The pairs of a block take 2^lgs systems
+// (fastest) of the same sites, whose links then come from L1, and the next
+// 32-site groups.  Bound by issue and latency (52% issue-active, 9,100
+// instructions per site and system, of which 1,728 products): 24^3 x 48, 8
+// systems, M: 2.38 ms, FP64 arithmetic 8.15 ms; 4^4, 16 systems 17.3 us against
+// 36.6 us (there one block's chain of instructions).  Measured beside it: one
+// thread per site unrolled over the hops, 2.43 ms and 21.7 us; the input
+// converted once by a pass of its own, 2.19 ms with the pass, 22 us.
+template <bool DAG, int EPI>
+__global__ void __launch_bounds__(128, 4) dslash_fx_kernel(const DslashArgs a, const int4* links_fx, int lgs) {
+  __shared__ longlong2 xch[4][3][32];
+  __shared__ unsigned xe[4][32][2];
+  __shared__ double xsum[4];
+  const Geom& g = a.g;
+  const int rg = blockIdx.x % a.rhs_groups;
+  const int sb = blockIdx.x / a.rhs_groups;
+  const int par = a.c.parity < 0 ? (sb & 1) : a.c.parity;
+  const int gb = a.c.parity < 0 ? (sb >> 1) : sb;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int sp = warp & 1, pair = warp >> 1;
+  const int grp = gb * (int)(blockDim.x >> (6 + lgs)) + (pair >> lgs);  // 32-site group
+  const int cb = grp * 32 + lane;
+  const int r = (rg << lgs) + (pair & ((1 << lgs) - 1));
+  const int nrhs = a.c.nrhs;
+  const bool act = r < nrhs && (a.c.active == nullptr || a.c.active[r] != 0) && cb < g.Vh;
+  if (a.trace_count && blockIdx.x == 0 && threadIdx.x == 0) {
+    int n = 0;
+    for (int q = 0; q < nrhs; ++q) n += (a.c.active == nullptr || a.c.active[q] != 0) ? 1 : 0;
+    *a.trace_count = n;
+  }
+  constexpr int SF = DAG ? +1 : -1;
+  FxSum t;
+  if (act) {
+    const Site s = site_of(g, par, cb);
+    const int opar = par ^ 1;
+    const size_t cs = (size_t)g.Vh;
+    const double2* fup = reinterpret_cast<const double2*>(a.c.in) + ((size_t)(r * 2 + opar) * 12 + 3 * sp) * cs;
+    t.E = kFxMinExp;
+    t.big = 0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) t.upr[c] = t.upi[c] = 0;
+#pragma unroll 1
+    for (int it = 0; it < 2; ++it) {
+      const int4* uf = links_fx + (size_t)(4 * it + par) * a.nwarp * 288;  // direction 2 it; the next one: + 576 nwarp
+      const int4* ub = links_fx + (size_t)(4 * it + opar) * a.nwarp * 288;
+      const double2* fdn = fup + (6 + 3 * (it ? 0 : 1 - 2 * sp)) * (ptrdiff_t)cs;
+      const int so = it && sp ? -1 : 1, se = it || sp ? 1 : -1;  // phase signs: i^ak = so i, se
+#pragma unroll
+      for (int c = 0; c < 3; ++c) t.lor[c] = t.loi[c] = 0;
+      {
+        const int c = it ? s.c[2] : s.c[0], L = it ? g.L[2] : g.L[0], st = it ? g.stride[2] : 1;
+        const int n1 = (c + 1 < L ? s.lex + st : s.lex - (L - 1) * st) >> 1;
+        const int n2 = (c > 0 ? s.lex - st : s.lex + (L - 1) * st) >> 1;
+        fx_hop<true, false>(t, fup + n1, fdn + n1, uf + fx_row(cb, 9), cs, SF * so >> 1, 0);
+        fx_hop<true, true>(t, fup + n2, fdn + n2, ub + fx_row(n2, 9), cs, -SF * so >> 1, 0);
+      }
+      // lower row: SF (-so i (w_f - w_b)_odd + se (w_f - w_b)_even); the sums are
+      // kept as the bracket times se
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const long long x = t.lor[c], y = t.loi[c];
+        t.lor[c] = so == se ? y : -y;
+        t.loi[c] = so == se ? -x : x;
+      }
+      {
+        const int c = it ? s.c[3] : s.c[1], L = it ? g.L[3] : g.L[1], st = it ? g.stride[3] : g.stride[1];
+        const int n1 = (c + 1 < L ? s.lex + st : s.lex - (L - 1) * st) >> 1;
+        const int n2 = (c > 0 ? s.lex - st : s.lex + (L - 1) * st) >> 1;
+        const size_t next = (size_t)a.nwarp * 576;
+        const bool ap = it && g.antiperiodic;
+        fx_hop<false, false>(t, fup + n1, fdn + n1, uf + next + fx_row(cb, 9), cs, SF * se >> 1,
+                             ap && c == L - 1 ? -1 : 0);
+        fx_hop<false, true>(t, fup + n2, fdn + n2, ub + next + fx_row(n2, 9), cs, -SF * se >> 1,
+                            ap && c == 0 ? -1 : 0);
+      }
+      if (it == 0) {  // row 1 - sp
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+          xch[warp][c][lane] = se > 0 ? make_longlong2(t.lor[c], t.loi[c]) : make_longlong2(-t.lor[c], -t.loi[c]);
+        xe[warp][lane][0] = t.E;
+      }
+    }
+    if ((t.big >> 20) > kFxMaxExp || (t.big != 0 && (t.big >> 20) < kFxMinExp)) t.E = kFxBad;
+    xe[warp][lane][1] = t.E;
+  }
+  __syncthreads();
+  double part = 0.0;
+  if (act) {
+    Cx<double> acc[6];
+    const unsigned Eo = xe[warp ^ 1][lane][0];
+    // the pair's common unit; kFxBad if either sum is out of range
+    const unsigned E = max(t.E, xe[warp ^ 1][lane][1]);
+    double unit = __hiloint2double((int)(E - 55u) << 20, 0);  // 2^(E - 1078)
+    if (E == kFxBad) {
+      Cx<double> all[12];
+      hop_sum_f64<DAG>(all, &a.g, a.links, a.c.in, r, par, cb);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        acc[c] = sp == 0 ? all[c] : all[3 + c];
+        acc[3 + c] = sp == 0 ? all[6 + c] : all[9 + c];
+      }
+      unit = 1.0;
+    } else {
+      const unsigned d = E - t.E, dd = E - Eo;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const longlong2 o = xch[warp ^ 1][c][lane];
+        const long long lr = shr64_s(t.lor[c], d) + shr64_s(o.x, dd), li = shr64_s(t.loi[c], d) + shr64_s(o.y, dd);
+        acc[c] = {(double)shr64_s(t.upr[c], d), (double)shr64_s(t.upi[c], d)};
+        acc[3 + c] = SF > 0 ? Cx<double>{(double)lr, (double)li} : Cx<double>{(double)-lr, (double)-li};
+      }
+    }
+    if constexpr (EPI == EPI_OUT) {
+      switch (2 * a.c.centre + (a.c.out_inv ? 1 : 0)) {
+        case 0: part = fx_epilogue<EPI, 0, false>(a, sp, r, par, cb, unit, acc); break;
+        case 1: part = fx_epilogue<EPI, 0, true>(a, sp, r, par, cb, unit, acc); break;
+        case 2: part = fx_epilogue<EPI, 1, false>(a, sp, r, par, cb, unit, acc); break;
+        case 3: part = fx_epilogue<EPI, 1, true>(a, sp, r, par, cb, unit, acc); break;
+        case 4: part = fx_epilogue<EPI, 2, false>(a, sp, r, par, cb, unit, acc); break;
+        default: part = fx_epilogue<EPI, 2, true>(a, sp, r, par, cb, unit, acc); break;
+      }
+    } else {  // the solver's operator (launch_one checks the form)
+      part = fx_epilogue<EPI, 2, false>(a, sp, r, par, cb, unit, acc);
+    }
+  }
+  if (EPI != EPI_OUT || a.c.partial != nullptr) {
+    const double ps = warp_sum(part);
+    if (lane == 0) xsum[warp] = ps;
+    __syncthreads();
+    if (lane == 0 && sp == 0 && r < nrhs && grp < a.nwarp)
+      a.c.partial[((size_t)r * 2 + par) * a.nwarp + grp] = xsum[warp] + xsum[warp + 1];
+  }
+}
+
+}  // namespace tml

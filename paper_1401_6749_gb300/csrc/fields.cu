@@ -256,6 +256,50 @@ __global__ void pack_links_kernel(Geom g, void* out, const double* U) {
   }
 }
 
+// canonical FP64 links -> fixed-point halves [mu][parity][group of 32 sites][9][32]: a part u as
+// round(u 2^54) = hi 2^27 + lo, |lo| <= 2^26, one complex number per 16 bytes
+// (re.hi, re.lo, im.hi, im.lo); *bad is set if a part exceeds 1.25 or is not
+// a number
+__device__ __forceinline__ int2 fx_link(double u, bool& bad) {
+  if (!(fabs(u) <= 1.25)) {
+    bad = true;
+    return make_int2(0, 0);
+  }
+  const long long q = __double2ll_rn(u * 18014398509481984.0);  // 2^54
+  const int lo = (int)((q + (1 << 26)) & ((1 << 27) - 1)) - (1 << 26);
+  return make_int2((int)((q - lo) >> 27), lo);
+}
+
+__global__ void pack_links_fx_kernel(Geom g, int4* out, const double* U, int* bad) {
+  const long V = 2L * g.Vh;
+  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= 4 * V) return;
+  const int mu = (int)(i / V);
+  const int lex = (int)(i % V);
+  const int x = lex % g.L[0], y = (lex / g.stride[1]) % g.L[1];
+  const int z = (lex / g.stride[2]) % g.L[2], t = lex / g.stride[3];
+  const int par = (x + y + z + t) & 1;
+  const double2* src = reinterpret_cast<const double2*>(U) + ((size_t)mu * V + lex) * 9;
+  const size_t cb = (size_t)(lex >> 1), nw = (size_t)((g.Vh + 31) >> 5);
+  int4* dst = out + ((size_t)(mu * 2 + par) * nw + (cb >> 5)) * 288 + (cb & 31);
+  bool b = false;
+#pragma unroll
+  for (int u = 0; u < 9; ++u) {
+    const double2 v = src[u];
+    const int2 re = fx_link(v.x, b), im = fx_link(v.y, b);
+    dst[u * 32] = make_int4(re.x, re.y, im.x, im.y);
+  }
+  if (b) atomicOr(bad, 1);
+}
+
+size_t links_fx_bytes(const Geom& g) { return 8 * (size_t)nwarp_of(g) * 288 * sizeof(int4); }
+
+tm_status_t pack_links_fx(const Geom& g, void* out, const double* U, int* bad, cudaStream_t s) {
+  pack_links_fx_kernel<<<blocks_for(4L * 2 * g.Vh, 256), 256, 0, s>>>(g, static_cast<int4*>(out), U, bad);
+  count_launch();
+  return check_launch("pack_links_fx");
+}
+
 template <class S, int RECON>
 static size_t link_bytes_t(const Geom& g) {
   using F = LinkFmt<S, RECON>;

@@ -1,0 +1,98 @@
+"""The FP64 Dslash with the fixed-point hopping sum against the FP64 oracle:
+ragged site groups and batches, steep and sparse fields, values out of the
+fixed point's range, and links that it does not take.
+
+Tolerance: every term of the sum errs by at most 2^-53 of the largest
+component met (inputs 2^-56, links 2^-55 of the factor, dropped products 2^-56,
+the oracle's own roundings 2^-53), 96 terms and the final FP64 operations
+together stay below 2^-46 of it, about 1.4e-14; typical L2 errors are 2e-16.
+"""
+import numpy as np
+import pytest
+import torch
+
+from .gpu_util import pack, require_gpu, site_shape, to_dev, unpack
+from oracle import operator as oop
+from paper_1401_6749_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+KAPPA, MU = 0.16, 0.01
+
+
+def _apply(tl, op, L, psi, **kw):
+    n = psi.shape[0]
+    f = pack(tl, L, psi, tl.F64)
+    out = torch.empty_like(f)
+    tl.tm_dslash(op, out, f, n, prec=tl.F64, **kw)
+    return unpack(tl, L, out, tl.F64, n)
+
+
+def _local_max(psi):
+    """Largest component of each site and its eight neighbours, (n, T, Z, Y, X)."""
+    m = np.maximum(np.abs(psi.real), np.abs(psi.imag)).max(axis=(-1, -2))
+    out = m.copy()
+    for ax in range(1, 5):
+        for s in (1, -1):
+            out = np.maximum(out, np.roll(m, s, axis=ax))
+    return out
+
+
+@pytest.mark.parametrize("L,n", [((2, 2, 2, 2), 1), ((4, 4, 4, 4), 5), ((6, 4, 2, 10), 3), ((10, 6, 8, 4), 2),
+                                 ((4, 6, 6, 34), 1)])
+@pytest.mark.parametrize("kw", [{}, {"dagger": True}, {"mu_zero": True}])
+def test_ragged(L, n, kw):
+    tl = require_gpu()
+    U = synth.gauge_field(L, 5)
+    op = tl.Operator(L, KAPPA, MU, to_dev(U))
+    psi = synth.random_spinor(L, n, 9)
+    got = _apply(tl, op, L, psi, **kw)
+    ref = oop.apply_M(U, psi, KAPPA, 0.0 if kw.get("mu_zero") else MU, dagger=bool(kw.get("dagger")))
+    assert np.linalg.norm(got - ref) <= 4e-16 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("decades", [3, 30, 250])
+def test_steep_fields(decades):
+    """Neighbouring sites of very unlike size: the error follows the largest
+    component of each stencil (beyond 2^-863 .. 2^878 the FP64 arithmetic)."""
+    tl = require_gpu()
+    L = (6, 4, 4, 8)
+    U = synth.gauge_field(L, 6)
+    op = tl.Operator(L, KAPPA, MU, to_dev(U))
+    rng = np.random.default_rng(3)
+    scale = 10.0 ** rng.uniform(-decades, decades, size=(2,) + site_shape(L))
+    scale[:, 1, :2] = 0.0  # zero sites among them
+    psi = synth.random_spinor(L, 2, 11) * scale[..., None, None]
+    got = _apply(tl, op, L, psi)
+    ref = oop.apply_M(U, psi, KAPPA, MU)
+    err = np.abs(got - ref).max(axis=(-1, -2))
+    assert np.all(err <= 1.5e-14 * _local_max(psi))
+
+
+def test_special_values():
+    """Infinities and NaN reach the sites that read them and no others."""
+    tl = require_gpu()
+    L = (4, 4, 4, 8)
+    U = synth.gauge_field(L, 7)
+    op = tl.Operator(L, KAPPA, MU, to_dev(U))
+    psi = synth.random_spinor(L, 3, 12)
+    clean = _apply(tl, op, L, psi)
+    bad = psi.copy()
+    bad[1, 2, 1, 0, 3, 1, 2] = np.inf
+    bad[2, 0, 3, 3, 3, 0, 0] = np.nan
+    got = _apply(tl, op, L, bad)
+    touched = ~np.isfinite(_local_max(np.nan_to_num(bad, nan=np.inf, posinf=np.inf)))
+    same = (got == clean).all(axis=(-1, -2))
+    assert same[~touched].all()
+    assert not np.isfinite(got[touched]).all(axis=(-1, -2)).any()
+
+
+def test_links_out_of_range():
+    """Links beyond the fixed point's range take the FP64 arithmetic."""
+    tl = require_gpu()
+    L = (4, 4, 4, 4)
+    U = synth.gauge_field(L, 8)
+    U[2, 1, 1, 1, 1] *= 40.0
+    op = tl.Operator(L, KAPPA, MU, to_dev(U), recon=18)
+    psi = synth.random_spinor(L, 2, 13)
+    ref = oop.apply_M(U, psi, KAPPA, MU)
+    assert np.linalg.norm(_apply(tl, op, L, psi) - ref) <= 1e-15 * np.linalg.norm(ref)
