@@ -43,26 +43,13 @@ __device__ __forceinline__ T warp_transpose_reduce(T (&v)[32]) {
 constexpr int kLocalK = 4;          // sites per thread
 constexpr int kLocalChunk = 256 * kLocalK;
 
-// momenta of a projected contraction: p = 2 pi (n_x / X, n_y / Y, n_z / Z)
-constexpr int kMaxMom = 64;
-struct MomList {
-  int n;
-  int p[kMaxMom][3];
-};
-
-// MOM: the site's R is multiplied by exp(-i p.x), block z = rhs * n + momentum
-template <class S, bool MOM = false>
+template <class S>
 __global__ void __launch_bounds__(256) local_partial_kernel(Geom g, const void* Lf, const void* Rf,
-                                                            int nchunk, double* partial,
-                                                            MomList mom = MomList{}) {
+                                                            int nchunk, double* partial) {
   using R = typename Prec<S>::R;
-  // MOM: the momentum is the fastest block index, so the blocks of one chunk
-  // (one set of sites) for all momenta run together and re-read L, R from L2
-  const int q = MOM ? (int)blockIdx.x % mom.n : 0;
-  const int chunk = MOM ? (int)blockIdx.x / mom.n : (int)blockIdx.x;
+  const int chunk = (int)blockIdx.x;
   const int t = blockIdx.y >> 1, par = blockIdx.y & 1;
   const int rhs = blockIdx.z;
-  const int slot_rhs = MOM ? rhs * mom.n + q : rhs;  // index of this contraction's output
   R acc[32];
 #pragma unroll
   for (int j = 0; j < 32; ++j) acc[j] = 0;
@@ -74,27 +61,6 @@ __global__ void __launch_bounds__(256) local_partial_kernel(Geom g, const void* 
       Cx<R> l[12], r[12];
       load_spinor<S>(l, Lf, b0, (size_t)g.Vh);
       load_spinor<S>(r, Rf, b0, (size_t)g.Vh);
-      if constexpr (MOM) {
-        const Site st = site_of(g, par, t * g.V3h + i);
-        // phase -2 pi sum_k n_k x_k / L_k, reduced exactly modulo one turn first
-        const long num = (long)((mom.p[q][0] * st.c[0]) % g.L[0]) * g.L[1] * g.L[2] +
-                         (long)((mom.p[q][1] * st.c[1]) % g.L[1]) * g.L[0] * g.L[2] +
-                         (long)((mom.p[q][2] * st.c[2]) % g.L[2]) * g.L[0] * g.L[1];
-        const long den = (long)g.L[0] * g.L[1] * g.L[2];
-        const double frac = (double)(num % den) / (double)den;
-        Cx<R> ph;
-        if constexpr (kWide<R>) {
-          double sn, cn;
-          sincospi(-2.0 * frac, &sn, &cn);
-          ph = {(R)cn, (R)sn};
-        } else {
-          float sn, cn;
-          sincospif(-2.0f * (float)frac, &sn, &cn);
-          ph = {cn, sn};
-        }
-#pragma unroll
-        for (int k = 0; k < 12; ++k) r[k] = ph * r[k];
-      }
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -115,9 +81,198 @@ __global__ void __launch_bounds__(256) local_partial_kernel(Geom g, const void* 
     double s = 0.0;
 #pragma unroll
     for (int w = 0; w < 8; ++w) s += sh[w][threadIdx.x];
-    const size_t slot = (((size_t)slot_rhs * g.L[3] + t) * 2 + par) * nchunk + chunk;
+    const size_t slot = (((size_t)rhs * g.L[3] + t) * 2 + par) * nchunk + chunk;
     partial[slot * 32 + threadIdx.x] = s;
   }
+}
+
+// ------------------------------------------- momentum-projected local loops
+// momenta p = 2 pi (n_x / X, n_y / Y, n_z / Z)
+constexpr int kMaxMom = 64;
+struct MomList {
+  int n;
+  int p[kMaxMom][3];
+};
+
+// The phases exp(-i p.x) of the sites of one slice, for both checkerboards of
+// (t + parity): [parity][i][nq] complex numbers, momenta q0 .. q0 + nq - 1 (zero
+// beyond the list).  The argument is reduced exactly modulo one turn first.
+template <class R>
+__global__ void mom_phase_kernel(Geom g, MomList mom, int q0, int nq, Cx<R>* ph) {
+  const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= 2L * g.V3h * nq) return;
+  const int q = q0 + (int)(k % nq);
+  const long pi = k / nq;
+  const Site st = site_of(g, (int)(pi / g.V3h), (int)(pi % g.V3h));
+  Cx<R> v = {(R)0, (R)0};
+  if (q < mom.n) {
+    // phase -2 pi sum_k n_k x_k / L_k
+    const long num = (long)((mom.p[q][0] * st.c[0]) % g.L[0]) * g.L[1] * g.L[2] +
+                     (long)((mom.p[q][1] * st.c[1]) % g.L[1]) * g.L[0] * g.L[2] +
+                     (long)((mom.p[q][2] * st.c[2]) % g.L[2]) * g.L[0] * g.L[1];
+    const long den = (long)g.L[0] * g.L[1] * g.L[2];
+    const double frac = (double)(num % den) / (double)den;
+    if constexpr (kWide<R>) {
+      double sn, cn;
+      sincospi(-2.0 * frac, &sn, &cn);
+      v = {(R)cn, (R)sn};
+    } else {
+      float sn, cn;
+      sincospif(-2.0f * (float)frac, &sn, &cn);
+      v = {cn, sn};
+    }
+  }
+  ph[k] = v;
+}
+
+// All momenta of a chunk of sites in one pass: a small complex matrix product
+// out[q][ab] = sum_x ph[q][x] m[x][ab] with the 16 bilinears
+// m_ab(x) = sum_c conj(L_ac) R_bc formed once per site.  Per tile of 128 sites
+// each thread forms one site's m and the block loads the tile's phases into
+// shared memory; then warp w takes the sites w, w + 4, ..., lane (qg, cg) the
+// momenta qg QT .. qg QT + QT - 1 and the bilinears 2 cg, 2 cg + 1.  FP32 sums run
+// over eight sites and are then added with compensation (two-sum), so their
+// error stays that of a short sum.  Bound by the FMA pipe (64 FMAs per site and
+// momentum); a pass per momentum, which it replaces, formed the 16 bilinears
+// and the phase again for each.
+constexpr int kMomTile = 128;
+template <class S, int QT>
+__global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const void* Lf, const void* Rf, int nchunk,
+                                                               const void* phases, int q0, int nmom, double* partial) {
+  using R = typename Prec<S>::R;
+  using O = Ar<R>;
+  extern __shared__ __align__(16) unsigned char mom_smem[];
+  Cx<R>* sm = reinterpret_cast<Cx<R>*>(mom_smem);  // [site][8 pairs, swizzled by site][2]
+  Cx<R>* sp = sm + kMomTile * 16;                  // [site][4 QT]
+  constexpr int nq = 4 * QT;
+  const int chunk = (int)blockIdx.x;
+  const int t = blockIdx.y >> 1, par = blockIdx.y & 1;
+  const int rhs = blockIdx.z;
+  const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
+  const int cg = lane & 7, qg = lane >> 3;
+  const Cx<R>* ph = static_cast<const Cx<R>*>(phases) + (size_t)((t + par) & 1) * g.V3h * nq;
+  Cx<R> acc[QT][2], err[QT][2];
+#pragma unroll
+  for (int j = 0; j < QT; ++j) acc[j][0] = acc[j][1] = err[j][0] = err[j][1] = {(R)0, (R)0};
+  const int iend = min(g.V3h, (chunk + 1) * kLocalChunk);
+#pragma unroll 1
+  for (int i0 = chunk * kLocalChunk; i0 < iend; i0 += kMomTile) {
+    const int i = i0 + (int)threadIdx.x;
+    Cx<R> m[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) m[k] = {(R)0, (R)0};
+    if (i < iend) {
+      const size_t b0 = SpinorRef<S>::base(g, rhs, par, t * g.V3h + i);
+      Cx<R> l[12], r[12];
+      load_spinor<S>(l, Lf, b0, (size_t)g.Vh);
+      load_spinor<S>(r, Rf, b0, (size_t)g.Vh);
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          R zr = (R)0, zi = (R)0;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const Cx<R> x = l[3 * a + c], y = r[3 * b + c];
+            zr = O::fma(x.re, y.re, zr);
+            zr = O::fma(x.im, y.im, zr);
+            zi = O::fma(x.re, y.im, zi);
+            zi = O::fma(-x.im, y.re, zi);
+          }
+          m[4 * a + b] = {O::norm(zr), O::norm(zi)};
+        }
+    }
+    __syncthreads();  // the previous tile has been read
+#pragma unroll
+    for (int k = 0; k < 16; ++k) sm[threadIdx.x * 16 + 2 * ((k >> 1) ^ (threadIdx.x & 7)) + (k & 1)] = m[k];
+    const int rows = min(kMomTile, iend - i0);
+    for (int k = threadIdx.x; k < rows * nq; k += kMomTile) sp[k] = ph[(size_t)i0 * nq + k];
+    __syncthreads();
+#pragma unroll 1
+    for (int s0 = wq; s0 < rows; s0 += 32) {
+      Cx<R> z[QT][2];
+#pragma unroll
+      for (int j = 0; j < QT; ++j) z[j][0] = z[j][1] = {(R)0, (R)0};
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int s = s0 + 4 * k;
+        if (s < rows) {
+          const Cx<R> m0 = sm[s * 16 + 2 * (cg ^ (s & 7))], m1 = sm[s * 16 + 2 * (cg ^ (s & 7)) + 1];
+#pragma unroll
+          for (int j = 0; j < QT; ++j) {
+            const Cx<R> p = sp[s * nq + qg * QT + j];
+            z[j][0] = {O::fma(-p.im, m0.im, O::fma(p.re, m0.re, z[j][0].re)), O::fma(p.im, m0.re, O::fma(p.re, m0.im, z[j][0].im))};
+            z[j][1] = {O::fma(-p.im, m1.im, O::fma(p.re, m1.re, z[j][1].re)), O::fma(p.im, m1.re, O::fma(p.re, m1.im, z[j][1].im))};
+          }
+        }
+      }
+      auto add = [](R& s, R& e, R v) {
+        if constexpr (std::is_same<R, float>::value) {
+          const FF f = ff_two_sum(s, v);
+          s = f.hi;
+          e = __fadd_rn(e, f.lo);
+        } else {
+          s = O::add(s, O::norm(v));
+        }
+      };
+#pragma unroll
+      for (int j = 0; j < QT; ++j)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          add(acc[j][c].re, err[j][c].re, z[j][c].re);
+          add(acc[j][c].im, err[j][c].im, z[j][c].im);
+        }
+    }
+  }
+  // the warps' sums, in order, in FP64
+  __syncthreads();
+  double* red = reinterpret_cast<double*>(mom_smem);  // [warp][q of the group][32]
+  static_assert(sizeof(double) * 4 * 32 * nq <= sizeof(Cx<R>) * kMomTile * (16 + nq), "the sums fit the tiles");
+#pragma unroll
+  for (int j = 0; j < QT; ++j)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      double* w = red + ((size_t)wq * nq + qg * QT + j) * 32 + 2 * (2 * cg + c);
+      w[0] = (double)acc[j][c].re + (double)err[j][c].re;
+      w[1] = (double)acc[j][c].im + (double)err[j][c].im;
+    }
+  __syncthreads();
+  for (int k = threadIdx.x; k < nq * 32; k += kMomTile) {
+    const int q = q0 + (k >> 5);
+    if (q >= nmom) continue;
+    double v = 0.0;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) v += red[(size_t)w * nq * 32 + k];
+    const size_t slot = ((((size_t)rhs * nmom + q) * g.L[3] + t) * 2 + par) * nchunk + chunk;
+    partial[slot * 32 + (k & 31)] = v;
+  }
+}
+
+// at most 32 momenta per pass: QT momenta per lane group
+constexpr int kMomPass = 32;
+static int mom_qt(int nq) {
+  const int q = (nq + 3) / 4;
+  return q <= 1 ? 1 : q <= 2 ? 2 : q <= 3 ? 3 : q <= 5 ? 5 : q <= 7 ? 7 : 8;
+}
+
+template <class S, int QT>
+static tm_status_t mom_launch(const Geom& g, const void* left, const void* right, int nrhs, const MomList& ml, int q0,
+                              void* phases, int nchunk, double* scratch, cudaStream_t s) {
+  using R = typename Prec<S>::R;
+  constexpr int nq = 4 * QT, smem = (int)sizeof(Cx<R>) * kMomTile * (16 + nq);
+  if (cudaFuncSetAttribute(mom_partial_kernel<S, QT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+      cudaSuccess) {
+    set_error("loop_contract_local_mom: %s", cudaGetErrorString(cudaGetLastError()));
+    return TM_ERR_CUDA;
+  }
+  const long np = 2L * g.V3h * nq;
+  mom_phase_kernel<R><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(g, ml, q0, nq, static_cast<Cx<R>*>(phases));
+  count_launch();
+  TM_TRY(check_launch("loop_contract_local_mom phases"));
+  const dim3 grid(nchunk, 2 * g.L[3], nrhs);
+  mom_partial_kernel<S, QT><<<grid, kMomTile, smem, s>>>(g, left, right, nchunk, phases, q0, ml.n, scratch);
+  count_launch();
+  return check_launch("loop_contract_local_mom");
 }
 
 // Gamma projection of a 4x4 complex matrix stored as 32 doubles (row-major, re/im).
@@ -626,18 +781,30 @@ extern "C" tm_status_t loop_contract_local_mom(const tm_geom_t* gg, const void* 
   tm_status_t st = scratch_alloc((void**)&scratch, local_scratch_bytes(g, n2), s);
   if (st != TM_OK) return st;
   const int nchunk = (g.V3h + kLocalChunk - 1) / kLocalChunk;
-  const dim3 grid(nchunk * n_mom, 2 * g.L[3], nrhs);
-  {
+  void* phases = nullptr;  // one pass of at most kMomPass momenta
+  const size_t cplx = prec == TM_PREC_F64 || prec == TM_PREC_FF ? 16 : 8;
+  const int nq_max = 4 * mom_qt(n_mom < kMomPass ? n_mom : kMomPass);
+  st = scratch_alloc(&phases, 2 * (size_t)g.V3h * nq_max * cplx, s);
+  if (st == TM_OK) {
     static const char* const kNames[kNumPrec] = {"localmom.f64", "localmom.f32", "localmom.f16", "localmom.bf16",
                                                   "localmom.ff"};
     TraceScope tr(s, prec_name(kNames, prec), 2.0 * 24.0 * prec_size(prec) * 2.0 * g.Vh, 0.0, n2);
-    st = by_prec_c(prec, [&](auto tag) {
-      using S = decltype(tag);
-      local_partial_kernel<S, true><<<grid, 256, 0, s>>>(g, left, right, nchunk, scratch, ml);
-      count_launch();
-      return check_launch("loop_contract_local_mom");
-    });
+    for (int q0 = 0; q0 < n_mom && st == TM_OK; q0 += kMomPass) {
+      const int qt = mom_qt(n_mom - q0 < kMomPass ? n_mom - q0 : kMomPass);
+      st = by_prec_c(prec, [&](auto tag) {
+        using S = decltype(tag);
+        switch (qt) {
+          case 1: return mom_launch<S, 1>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s);
+          case 2: return mom_launch<S, 2>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s);
+          case 3: return mom_launch<S, 3>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s);
+          case 5: return mom_launch<S, 5>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s);
+          case 7: return mom_launch<S, 7>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s);
+          default: return mom_launch<S, 8>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s);
+        }
+      });
+    }
   }
+  dev_free(phases, s);
   if (st == TM_OK) {
     local_final_kernel<<<dim3(g.L[3], n2), 32, 0, s>>>(scratch, nchunk, g.L[3], gamma_tab(),
                                                         mode != TM_LOOP_STD, out);

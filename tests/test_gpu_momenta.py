@@ -1,0 +1,55 @@
+"""Momentum-projected local loops, all momenta of a pass in one kernel: at the
+edges of the momentum groups (4, 8, ..., 32 per pass) and of the site tiles (128)
+and chunks (1024), against the FP64 oracle.
+
+Tolerance: an output sums 4 phased bilinears per site.  In FP32 a bilinear of
+three complex products errs by at most 7 u sum_c |L||R|, its phase by 4 u, a sum of
+eight sites by 8 u (longer sums are compensated), u = 2^-24: 24 u of
+sum |L||R| covers it, and 24 2^-46 the float-float arithmetic, whose steps err by
+a few 2^-47."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import loops as olo
+from paper_1401_6749_gb300 import synth
+
+from .gpu_util import from_dev, pack, require_gpu, unpack
+
+pytestmark = pytest.mark.gpu
+U = {"f16": 2.0 ** -24, "bf16": 2.0 ** -24, "f32": 2.0 ** -24, "ff": 2.0 ** -46, "f64": 2.0 ** -50}
+
+
+def _momenta(n):
+    rng = np.random.default_rng(n)
+    return np.concatenate([[[0, 0, 0]], rng.integers(-9, 10, size=(n - 1, 3))])
+
+
+def _check(L, n, nmom, prec, mode):
+    tl = require_gpu()
+    p = tl.PREC[prec]
+    fl, fr = (pack(tl, L, synth.random_spinor(L, n, s), p) for s in (4, 5))
+    left, right = (unpack(tl, L, f, p, n) for f in (fl, fr))  # the stored values
+    mom = _momenta(nmom)
+    out = torch.full((n, nmom, 16, L[3], 2), float("nan"), dtype=torch.float64, device="cuda")
+    tl.loop_contract_local_mom(L, fl, fr, p, n, tl.LOOP_MODE[mode], mom, out)
+    got = from_dev(out, (n, nmom, 16, L[3]))
+    ref = olo.local_loops_mom(left, right, mode, mom)
+    size = np.einsum("ntzyxac,ntzyxbc->nt", np.abs(left), np.abs(right))[:, None, None, :]
+    assert np.all(np.abs(got - ref) <= 24 * U[prec] * size)
+
+
+@pytest.mark.parametrize("nmom", [1, 4, 5, 8, 12, 13, 20, 21, 28, 29, 32, 33, 64])
+def test_momentum_groups(nmom):
+    _check((6, 4, 8, 4), 2, nmom, "f32", "vv")
+
+
+@pytest.mark.parametrize("L", [(2, 2, 2, 2), (8, 8, 4, 2), (10, 6, 10, 4), (16, 12, 12, 2), (16, 16, 10, 4)])
+@pytest.mark.parametrize("prec", ["f16", "bf16", "f32", "ff", "f64"])
+def test_site_tiles(L, prec):
+    _check(L, 1, 7, prec, "std")
+
+
+@pytest.mark.parametrize("prec", ["ff", "f64"])
+def test_wide_full_pass(prec):
+    _check((6, 4, 8, 4), 1, 32, prec, "gen")
