@@ -43,9 +43,35 @@ __device__ __forceinline__ T warp_transpose_reduce(T (&v)[32]) {
 constexpr int kLocalK = 4;          // sites per thread
 constexpr int kLocalChunk = 256 * kLocalK;
 
-template <class S>
+// one momentum p = 2 pi (n_x / X, n_y / Y, n_z / Z), 0 <= n < extent
+struct Mom3 {
+  int p[3];
+};
+
+// exp(-i p.x) at a site; the argument is reduced exactly modulo one turn first
+template <class R>
+__device__ __forceinline__ Cx<R> mom_phase(const Geom& g, const Mom3& q, const Site& st) {
+  // phase -2 pi sum_k n_k x_k / L_k
+  const long num = (long)((q.p[0] * st.c[0]) % g.L[0]) * g.L[1] * g.L[2] +
+                   (long)((q.p[1] * st.c[1]) % g.L[1]) * g.L[0] * g.L[2] +
+                   (long)((q.p[2] * st.c[2]) % g.L[2]) * g.L[0] * g.L[1];
+  const long den = (long)g.L[0] * g.L[1] * g.L[2];
+  const double frac = (double)(num % den) / (double)den;
+  if constexpr (kWide<R>) {
+    double sn, cn;
+    sincospi(-2.0 * frac, &sn, &cn);
+    return {(R)cn, (R)sn};
+  } else {
+    float sn, cn;
+    sincospif(-2.0f * (float)frac, &sn, &cn);
+    return {cn, sn};
+  }
+}
+
+// MOM: the site's R is multiplied by exp(-i p.x) (a single non-zero momentum)
+template <class S, bool MOM = false>
 __global__ void __launch_bounds__(256) local_partial_kernel(Geom g, const void* Lf, const void* Rf,
-                                                            int nchunk, double* partial) {
+                                                            int nchunk, double* partial, Mom3 mom = Mom3{}) {
   using R = typename Prec<S>::R;
   const int chunk = (int)blockIdx.x;
   const int t = blockIdx.y >> 1, par = blockIdx.y & 1;
@@ -61,6 +87,11 @@ __global__ void __launch_bounds__(256) local_partial_kernel(Geom g, const void* 
       Cx<R> l[12], r[12];
       load_spinor<S>(l, Lf, b0, (size_t)g.Vh);
       load_spinor<S>(r, Rf, b0, (size_t)g.Vh);
+      if constexpr (MOM) {
+        const Cx<R> ph = mom_phase<R>(g, mom, site_of(g, par, t * g.V3h + i));
+#pragma unroll
+        for (int k = 0; k < 12; ++k) r[k] = ph * r[k];
+      }
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -87,41 +118,23 @@ __global__ void __launch_bounds__(256) local_partial_kernel(Geom g, const void* 
 }
 
 // ------------------------------------------- momentum-projected local loops
-// momenta p = 2 pi (n_x / X, n_y / Y, n_z / Z)
 constexpr int kMaxMom = 64;
 struct MomList {
   int n;
-  int p[kMaxMom][3];
+  Mom3 q[kMaxMom];
 };
 
 // The phases exp(-i p.x) of the sites of one slice, for both checkerboards of
 // (t + parity): [parity][i][nq] complex numbers, momenta q0 .. q0 + nq - 1 (zero
-// beyond the list).  The argument is reduced exactly modulo one turn first.
+// beyond the list).
 template <class R>
 __global__ void mom_phase_kernel(Geom g, MomList mom, int q0, int nq, Cx<R>* ph) {
   const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= 2L * g.V3h * nq) return;
   const int q = q0 + (int)(k % nq);
   const long pi = k / nq;
-  const Site st = site_of(g, (int)(pi / g.V3h), (int)(pi % g.V3h));
   Cx<R> v = {(R)0, (R)0};
-  if (q < mom.n) {
-    // phase -2 pi sum_k n_k x_k / L_k
-    const long num = (long)((mom.p[q][0] * st.c[0]) % g.L[0]) * g.L[1] * g.L[2] +
-                     (long)((mom.p[q][1] * st.c[1]) % g.L[1]) * g.L[0] * g.L[2] +
-                     (long)((mom.p[q][2] * st.c[2]) % g.L[2]) * g.L[0] * g.L[1];
-    const long den = (long)g.L[0] * g.L[1] * g.L[2];
-    const double frac = (double)(num % den) / (double)den;
-    if constexpr (kWide<R>) {
-      double sn, cn;
-      sincospi(-2.0 * frac, &sn, &cn);
-      v = {(R)cn, (R)sn};
-    } else {
-      float sn, cn;
-      sincospif(-2.0f * (float)frac, &sn, &cn);
-      v = {cn, sn};
-    }
-  }
+  if (q < mom.n) v = mom_phase<R>(g, mom.q[q], site_of(g, (int)(pi / g.V3h), (int)(pi % g.V3h)));
   ph[k] = v;
 }
 
@@ -260,8 +273,9 @@ static tm_status_t mom_launch(const Geom& g, const void* left, const void* right
                               void* phases, int nchunk, double* scratch, cudaStream_t s) {
   using R = typename Prec<S>::R;
   constexpr int nq = 4 * QT, smem = (int)sizeof(Cx<R>) * kMomTile * (16 + nq);
-  if (cudaFuncSetAttribute(mom_partial_kernel<S, QT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
-      cudaSuccess) {
+  if (smem > 48 * 1024 &&
+      cudaFuncSetAttribute(mom_partial_kernel<S, QT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+          cudaSuccess) {
     set_error("loop_contract_local_mom: %s", cudaGetErrorString(cudaGetLastError()));
     return TM_ERR_CUDA;
   }
@@ -375,6 +389,19 @@ __device__ __forceinline__ void load_spins2(Cx<typename Prec<S>::R> (&v)[6], con
   }
 }
 
+// float-float link U (adj: U^dag; neg: negated) whose first 16-byte unit is b0,
+// unit stride cs
+__device__ __forceinline__ void load_link9(Cx<FF> (&u)[9], const void* links, size_t b0, size_t cs, int adj, bool neg) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const float4 q = reinterpret_cast<const float4*>(links)[b0 + (size_t)(adj ? 3 * d + c : 3 * c + d) * cs];
+      const Cx<FF> v = {FF{q.x, q.y}, FF{q.z, q.w}};
+      u[3 * c + d] = {neg ? -v.re : v.re, (adj != 0) != neg ? -v.im : v.im};
+    }
+}
+
 // w (+/-)= U r or U^dag r for two spins (four FMAs per complex multiply-add)
 template <bool ADJ, bool SUB, class R>
 __device__ __forceinline__ void link_times2(Cx<R> (&w)[6], const Mat3<R>& U, const Cx<R> (&r)[6]) {
@@ -408,6 +435,9 @@ __device__ __forceinline__ void outer_acc2(R (&acc)[16], const void* Lf, size_t 
 #pragma unroll
   for (int j = 0; j < 6; ++j) ws[j] = {sgn * w[j].re, sgn * w[j].im};
   if constexpr (kWide<R>) {
+    // the current row's sums are always acc[0..3]: a rotation of the sums per row
+    // instead of four copies of the code (or a run-time index, which would move
+    // acc to local memory)
 #pragma unroll 1
     for (int a = 0; a < 4; ++a) {
       Cx<R> l[3];
@@ -421,24 +451,24 @@ __device__ __forceinline__ void outer_acc2(R (&acc)[16], const void* Lf, size_t 
           l[c] = {FF{d.x, d.y}, FF{d.z, d.w}};
         }
       }
-      // a runtime index into acc would move it to local memory: select instead
+      R z[4];
 #pragma unroll
-      for (int aa = 0; aa < 4; ++aa) {
-        if (aa != a) continue;
+      for (int bb = 0; bb < 2; ++bb) {
+        R mr = acc[2 * bb], mi = acc[2 * bb + 1];
 #pragma unroll
-        for (int bb = 0; bb < 2; ++bb) {
-          R mr = acc[2 * (2 * aa + bb)], mi = acc[2 * (2 * aa + bb) + 1];
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            mr = O::fma(l[c].re, ws[3 * bb + c].re, mr);
-            mr = O::fma(l[c].im, ws[3 * bb + c].im, mr);
-            mi = O::fma(l[c].re, ws[3 * bb + c].im, mi);
-            mi = O::fma(-l[c].im, ws[3 * bb + c].re, mi);
-          }
-          acc[2 * (2 * aa + bb)] = mr;
-          acc[2 * (2 * aa + bb) + 1] = mi;
+        for (int c = 0; c < 3; ++c) {
+          mr = O::fma(l[c].re, ws[3 * bb + c].re, mr);
+          mr = O::fma(l[c].im, ws[3 * bb + c].im, mr);
+          mi = O::fma(l[c].re, ws[3 * bb + c].im, mi);
+          mi = O::fma(-l[c].im, ws[3 * bb + c].re, mi);
         }
+        z[2 * bb] = mr;
+        z[2 * bb + 1] = mi;
       }
+#pragma unroll
+      for (int j = 0; j < 12; ++j) acc[j] = acc[j + 4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[12 + j] = z[j];
     }
   } else {
     Cx<R> l[12];
@@ -531,6 +561,48 @@ __global__ void __launch_bounds__(256, oned_min_blocks<S>()) oneD_partial_kernel
         load_spins2_raw<S>(x, Rf, bx, cs, h);
         link_times2_raw<true, false, S>(w, u, x);
         outer_acc2<S>(acc, Lf, bf, cs, w, -sf);
+      }
+    } else if constexpr (std::is_same<R, FF>::value) {
+      // Float-float: both terms of a direction, spatial or temporal, run through
+      // one copy of the link and of the outer product (term 0: U_mu(x) R(x+mu);
+      // term 1: U_mu(x-mu)^dag R(x-mu), or U_t(x)^dag R(x) in time).  Unrolled over
+      // the terms and the two cases the code (a multiply-add is 12 instructions)
+      // exceeds the instruction cache: 54% issue-active, most stalls waiting for
+      // instructions, 8.65 ms at 24^3 x 48 with 8 systems; now 66-73%, 6.5 ms, bound
+      // by FP32 issue.  (FP64 is bound by its own pipe and keeps the unrolled form.)
+      using O = Ar<R>;
+      const bool time = mu == 3;
+      const R sf = (time && g.antiperiodic && cmu == Lmu - 1) ? (R)-1 : (R)1;
+      const int lb = (cmu > 0 ? s.lex - smu : s.lex + (Lmu - 1) * smu) >> 1;
+#pragma unroll
+      for (int j = 0; j < 6; ++j) w[j] = {(R)0, (R)0};
+#pragma unroll 1
+      for (int term = 0; term < 2; ++term) {
+        const bool back = term && !time;  // the link and site behind x
+        const size_t b0 = ((size_t)(mu * 2 + (back ? opar : par)) * 9) * cs + (back ? lb : cb);
+        Cx<R> u[9], r[6];
+        load_link9(u, links, b0, cs, term, back);
+        load_spins2<S>(r, Rf, !term ? bf : time ? bx : SpinorRef<S>::base(g, rhs, opar, lb), cs, h);
+        if (term && time) {
+#pragma unroll
+          for (int j = 0; j < 6; ++j) w[j] = {(R)0, (R)0};
+        }
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            R zr = w[3 * a + c].re, zi = w[3 * a + c].im;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+              const Cx<R> x = r[3 * a + d], y = u[3 * c + d];
+              zr = O::fma(y.re, x.re, zr);
+              zr = O::fma(-y.im, x.im, zr);
+              zi = O::fma(y.re, x.im, zi);
+              zi = O::fma(y.im, x.re, zi);
+            }
+            w[3 * a + c] = {O::norm(zr), O::norm(zi)};
+          }
+        if (time || term) outer_acc2<S>(acc, Lf, term && time ? bf : bx, cs, w, time ? (term ? -sf : sf) : (R)1);
       }
     } else {
       Cx<R> r[6];
@@ -774,37 +846,50 @@ extern "C" tm_status_t loop_contract_local_mom(const tm_geom_t* gg, const void* 
   for (int q = 0; q < n_mom; ++q)
     for (int k = 0; k < 3; ++k) {
       const int Lk = g.L[k];
-      ml.p[q][k] = ((mom[3 * q + k] % Lk) + Lk) % Lk;  // p and p + L are the same momentum
+      ml.q[q].p[k] = ((mom[3 * q + k] % Lk) + Lk) % Lk;  // p and p + L are the same momentum
     }
   const int n2 = nrhs * n_mom;
-  double* scratch = nullptr;
-  tm_status_t st = scratch_alloc((void**)&scratch, local_scratch_bytes(g, n2), s);
-  if (st != TM_OK) return st;
   const int nchunk = (g.V3h + kLocalChunk - 1) / kLocalChunk;
-  void* phases = nullptr;  // one pass of at most kMomPass momenta
-  const size_t cplx = prec == TM_PREC_F64 || prec == TM_PREC_FF ? 16 : 8;
+  // several momenta: the table of phases of one pass behind the partial sums
+  const size_t part = local_scratch_bytes(g, n2), cplx = prec == TM_PREC_F64 || prec == TM_PREC_FF ? 16 : 8;
   const int nq_max = 4 * mom_qt(n_mom < kMomPass ? n_mom : kMomPass);
-  st = scratch_alloc(&phases, 2 * (size_t)g.V3h * nq_max * cplx, s);
-  if (st == TM_OK) {
+  double* scratch = nullptr;
+  tm_status_t st = scratch_alloc((void**)&scratch, part + (n_mom > 1 ? 2 * (size_t)g.V3h * nq_max * cplx : 0), s);
+  if (st != TM_OK) return st;
+  void* phases = reinterpret_cast<char*>(scratch) + part;
+  {
     static const char* const kNames[kNumPrec] = {"localmom.f64", "localmom.f32", "localmom.f16", "localmom.bf16",
                                                   "localmom.ff"};
     TraceScope tr(s, prec_name(kNames, prec), 2.0 * 24.0 * prec_size(prec) * 2.0 * g.Vh, 0.0, n2);
-    for (int q0 = 0; q0 < n_mom && st == TM_OK; q0 += kMomPass) {
-      const int qt = mom_qt(n_mom - q0 < kMomPass ? n_mom - q0 : kMomPass);
-      st = by_prec_c(prec, [&](auto tag) {
-        using S = decltype(tag);
-        switch (qt) {
-          case 1: return mom_launch<S, 1>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s);
-          case 2: return mom_launch<S, 2>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s);
-          case 3: return mom_launch<S, 3>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s);
-          case 5: return mom_launch<S, 5>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s);
-          case 7: return mom_launch<S, 7>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s);
-          default: return mom_launch<S, 8>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s);
+    st = by_prec_c(prec, [&](auto tag) {
+      using S = decltype(tag);
+      if (n_mom == 1) {
+        // one momentum needs no table: 404 us at 24^3 x 48, FP32, 12 systems, against
+        // 434 us by the table and the matrix product; zero momentum, no phase
+        const dim3 grid(nchunk, 2 * g.L[3], nrhs);
+        const Mom3& q = ml.q[0];
+        if (q.p[0] || q.p[1] || q.p[2])
+          local_partial_kernel<S, true><<<grid, 256, 0, s>>>(g, left, right, nchunk, scratch, q);
+        else
+          local_partial_kernel<S><<<grid, 256, 0, s>>>(g, left, right, nchunk, scratch);
+        count_launch();
+        return check_launch("loop_contract_local_mom");
+      }
+      for (int q0 = 0; q0 < n_mom; q0 += kMomPass) {
+        tm_status_t ps;
+        switch (mom_qt(n_mom - q0 < kMomPass ? n_mom - q0 : kMomPass)) {
+          case 1: ps = mom_launch<S, 1>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s); break;
+          case 2: ps = mom_launch<S, 2>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s); break;
+          case 3: ps = mom_launch<S, 3>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s); break;
+          case 5: ps = mom_launch<S, 5>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s); break;
+          case 7: ps = mom_launch<S, 7>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s); break;
+          default: ps = mom_launch<S, 8>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s); break;
         }
-      });
-    }
+        if (ps != TM_OK) return ps;
+      }
+      return TM_OK;
+    });
   }
-  dev_free(phases, s);
   if (st == TM_OK) {
     local_final_kernel<<<dim3(g.L[3], n2), 32, 0, s>>>(scratch, nchunk, g.L[3], gamma_tab(),
                                                         mode != TM_LOOP_STD, out);

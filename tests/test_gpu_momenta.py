@@ -25,12 +25,12 @@ def _momenta(n):
     return np.concatenate([[[0, 0, 0]], rng.integers(-9, 10, size=(n - 1, 3))])
 
 
-def _check(L, n, nmom, prec, mode):
+def _check(L, n, nmom, prec, mode, mom=None):
     tl = require_gpu()
     p = tl.PREC[prec]
     fl, fr = (pack(tl, L, synth.random_spinor(L, n, s), p) for s in (4, 5))
     left, right = (unpack(tl, L, f, p, n) for f in (fl, fr))  # the stored values
-    mom = _momenta(nmom)
+    mom = _momenta(nmom) if mom is None else mom
     out = torch.full((n, nmom, 16, L[3], 2), float("nan"), dtype=torch.float64, device="cuda")
     tl.loop_contract_local_mom(L, fl, fr, p, n, tl.LOOP_MODE[mode], mom, out)
     got = from_dev(out, (n, nmom, 16, L[3]))
@@ -53,3 +53,9 @@ def test_site_tiles(L, prec):
 @pytest.mark.parametrize("prec", ["ff", "f64"])
 def test_wide_full_pass(prec):
     _check((6, 4, 8, 4), 1, 32, prec, "gen")
+
+
+@pytest.mark.parametrize("p", [(0, 0, 0), (3, -1, 2)])
+@pytest.mark.parametrize("prec", ["f16", "f32", "ff", "f64"])
+def test_single_momentum(p, prec):
+    _check((8, 6, 4, 6), 2, 1, prec, "vv", np.array([p]))
