@@ -727,6 +727,7 @@ __global__ void __launch_bounds__(128, (dslash_min_blocks<S, NR>())) dslash_kern
 }  // namespace tml
 
 #include "dslash_fx.cuh"
+#include "dslash_ffhalf.cuh"
 #include "dslash_x2.cuh"
 #include "dslash_mma.cuh"
 
@@ -734,8 +735,9 @@ namespace tml {
 
 // X2: two systems per thread in packed FP32x2 arithmetic (FP16/BF16, NR = 2);
 // MMA: the tensor-core kernel (FP16/BF16 with 18-real links, NR and bx unused)
-// FX: the fixed-point hopping sum (FP64 with links in range)
-template <class S, int RECON, bool DAG, int EPI, int NR, bool X2 = false, bool MMA = false, bool FX = false>
+// HALF: two warps per 32 sites, one per upper spin: FP64 with links in range
+// (fixed-point hopping sum) and float-float
+template <class S, int RECON, bool DAG, int EPI, int NR, bool X2 = false, bool MMA = false, bool HALF = false>
 tm_status_t launch_one(const tm_op* op, const DslashCall& c, cudaStream_t st, int bx = 128) {
   DslashArgs a;
   a.g = op->g;
@@ -769,7 +771,7 @@ tm_status_t launch_one(const tm_op* op, const DslashCall& c, cudaStream_t st, in
     }
   }
   int lgs = 0;
-  if constexpr (FX) {
+  if constexpr (HALF) {
     // pairs of warps, two to a block; where there are too few for every SM,
     // one to a block
     const long pairs = (long)a.nwarp * (c.parity < 0 ? 2 : 1) * c.nrhs;
@@ -804,7 +806,9 @@ tm_status_t launch_one(const tm_op* op, const DslashCall& c, cudaStream_t st, in
   const double fixed = 4.0 * 2.0 * op->g.Vh * link_reals * e;
   cudaEvent_t ev = nullptr;
   a.trace_count = trace_begin(st, &ev);
-  if constexpr (FX) dslash_fx_kernel<DAG, EPI><<<grid, bx, 0, st>>>(a, static_cast<const int4*>(op->links_fx), lgs);
+  if constexpr (HALF && std::is_same<S, double>::value)
+    dslash_fx_kernel<DAG, EPI><<<grid, bx, 0, st>>>(a, static_cast<const int4*>(op->links_fx), lgs);
+  else if constexpr (HALF) dslash_ff_kernel<DAG, EPI><<<grid, bx, 0, st>>>(a, lgs);
   else if constexpr (MMA) dslash_kernel_mma<S, DAG, EPI><<<grid, kMmaThreads, kMmaSmem, st>>>(a);
   else if constexpr (X2) dslash_kernel_x2<S, RECON, DAG, EPI><<<grid, bx, 0, st>>>(a);
   else dslash_kernel<S, RECON, DAG, EPI, NR><<<grid, bx, 0, st>>>(a);
@@ -878,8 +882,10 @@ tm_status_t launch_nr(const tm_op* op, const DslashCall& c, cudaStream_t st) {
       const bool form = EPI == EPI_OUT || !c.custom || (c.centre == 2 && !c.out_inv);
       if (op->links_fx && form) return launch_one<S, RECON, DAG, EPI, 1, false, false, true>(op, c, st);
     }
-    // FP64 with links out of the fixed point's range, and float-float:
-    // arithmetic-bound and register-heavy, one system per thread
+    if constexpr (std::is_same<S, FFloat>::value && EPI != EPI_CGUPD)
+      return launch_one<S, RECON, DAG, EPI, 1, false, false, true>(op, c, st);
+    // FP64 with links out of the fixed point's range: arithmetic-bound, one
+    // system per thread
     return launch_one<S, RECON, DAG, EPI, 1>(op, c, st);
   } else {
     if constexpr (kRawLinks<S, RECON>) {
