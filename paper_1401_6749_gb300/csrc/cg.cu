@@ -8,7 +8,8 @@
 // Per iteration (PLAIN, every vector in one precision):
 //   t = M p                       Dslash, fused |t|^2 per-warp partials
 //   alpha = |r|^2 / |t|^2         fixed-order reduction + scalar kernel
-//   r -= alpha M^dag t, x += alpha p   Dslash with fused update, |r|^2 partials
+//   r -= alpha M^dag t, x += alpha p   Dslash with fused update, |r|^2 partials (on
+//                                  the interleaved layout x moves with p below)
 //   beta = |r_new|^2 / |r|^2      fixed-order reduction + scalar kernel
 //   p = r + beta p
 // MIXED adds FP64 reliable updates (Sleijpen & van der Vorst): the iteration
@@ -171,7 +172,10 @@ __global__ void cg_alpha_kernel(CgState st, CgScalars sc) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= sc.nrhs) return;
   st.ru[i] = 0;  // the reliable update of the previous iteration is complete
-  if (!st.active[i]) return;
+  if (!st.active[i]) {
+    st.alpha[i] = 0.0;  // no step: il_xpay leaves x alone
+    return;
+  }
   const double pap = st.red[i];
   if (!isfinite(pap) || !(pap > 0.0)) {
     st.status[i] = TM_ERR_NAN;
@@ -298,17 +302,33 @@ static tm_status_t scalar_launch(void (*k)(CgState, CgScalars), const CgState& s
   return check_launch("cg scalar kernel");
 }
 
-static tm_status_t memcpy_d2d(void* dst, const void* src, size_t n, cudaStream_t s) {
-  if (cudaMemcpyAsync(dst, src, n, cudaMemcpyDeviceToDevice, s) != cudaSuccess) {
-    set_error("tm_cg_solve: device copy failed: %s", cudaGetErrorString(cudaGetLastError()));
-    return TM_ERR_CUDA;
-  }
-  return TM_OK;
-}
+// The planes of parities par0 .. par0 + npar - 1 of `rows` fields (or blocks of
+// interleaved fields) of `field` bytes each
+struct Half {
+  size_t field;
+  int rows, par0, npar;
+};
 
-static tm_status_t memset_d(void* dst, size_t n, cudaStream_t s) {
-  if (cudaMemsetAsync(dst, 0, n, s) != cudaSuccess) {
-    set_error("tm_cg_solve: memset failed: %s", cudaGetErrorString(cudaGetLastError()));
+// one 2-D operation, or one per row where the row pitch exceeds what that takes
+// (2^31 - 1 bytes); both parities are one contiguous range
+static tm_status_t half_op(void* dst, const void* src, const Half& h, cudaStream_t s) {
+  const size_t off = h.field / 2 * h.par0, width = h.field / 2 * h.npar;
+  char* d = (char*)dst + off;
+  const char* q = (const char*)src + off;
+  cudaError_t e = cudaSuccess;
+  if (h.npar == 2) {
+    e = src ? cudaMemcpyAsync(d, q, h.field * h.rows, cudaMemcpyDeviceToDevice, s)
+            : cudaMemsetAsync(d, 0, h.field * h.rows, s);
+  } else if (h.field <= 0x7fffffffu) {
+    e = src ? cudaMemcpy2DAsync(d, h.field, q, h.field, width, (size_t)h.rows, cudaMemcpyDeviceToDevice, s)
+            : cudaMemset2DAsync(d, h.field, 0, width, (size_t)h.rows, s);
+  } else {
+    for (int i = 0; i < h.rows && e == cudaSuccess; ++i)
+      e = src ? cudaMemcpyAsync(d + i * h.field, q + i * h.field, width, cudaMemcpyDeviceToDevice, s)
+              : cudaMemsetAsync(d + i * h.field, 0, width, s);
+  }
+  if (e != cudaSuccess) {
+    set_error("tm_cg_solve: device %s failed: %s", src ? "copy" : "memset", cudaGetErrorString(cudaGetLastError()));
     return TM_ERR_CUDA;
   }
   return TM_OK;
@@ -411,7 +431,8 @@ tm_status_t CgRun::setup() {
       if (ru_ff) { xff = c.take(F64); bff = c.take(F64); }
       y = c.take(F); r = c.take(F); p = c.take(F); t = c.take(F);
     } else {
-      b = c.take(F); r = c.take(F); p = c.take(F); t = c.take(F);
+      r = c.take(F); p = c.take(F); t = c.take(F);
+      b = prm.true_residual ? c.take(F) : r;  // only the true residual needs b again
       if (il) {
         eta_il = x_is_il ? const_cast<void*>(eta) : c.take(F);
         x_il = x_is_il ? x : c.take(F);
@@ -471,19 +492,23 @@ tm_status_t CgRun::setup() {
     TM_TRY(reduce());
     TM_TRY(scalar_launch(cg_init_kernel, st, sc, s));
   }
+  // vectors are initialised on the parities they live on (the other half of a
+  // Schur solve's is scratch)
+  const Half hl = {F / (il ? (size_t)((nrhs + 15) / 16) : (size_t)nrhs), il ? (nrhs + 15) / 16 : nrhs, par0, npar};
   if (mixed) {
+    const Half h64 = {F64 / (size_t)nrhs, nrhs, par0, npar};
     TM_TRY(rescale(g, lo, r, b64, st.sigma, nullptr, nullptr, nullptr, nrhs, par0, npar, s));
-    TM_TRY(memset_d(x, F64, s));
-    TM_TRY(memset_d(y, F, s));
+    TM_TRY(half_op(x, nullptr, h64, s));
+    TM_TRY(half_op(y, nullptr, hl, s));
     if (ru_ff) {
       TM_TRY(convert_masked(g, bff, TM_PREC_FF, b64, TM_PREC_F64, nrhs, nullptr, s));
-      TM_TRY(memset_d(xff, F64, s));
+      TM_TRY(half_op(xff, nullptr, h64, s));
     }
   } else {
-    TM_TRY(memcpy_d2d(r, b, F, s));
-    TM_TRY(memset_d(xs, F, s));
+    if (b != r) TM_TRY(half_op(r, b, hl, s));
+    TM_TRY(half_op(xs, nullptr, hl, s));
   }
-  TM_TRY(memcpy_d2d(p, r, F, s));
+  TM_TRY(half_op(p, r, hl, s));
   return TM_OK;
 }
 
@@ -515,7 +540,7 @@ tm_status_t CgRun::iteration() {
     TM_TRY(scalar_launch(cg_ru_kernel, st, sc, s));
     TM_TRY(rescale(g, lo, r, r64, st.sigma, p, st.ratio, st.ru, nrhs, par0, npar, s, ru_ff));
   }
-  if (il) return il_xpay(g, lo, p, r, st.beta, st.active, nrhs, par0, npar, s);
+  if (il) return il_xpay(g, lo, xs, p, r, st.alpha, st.beta, st.active, nrhs, par0, npar, s);
   return xpay(g, lo, p, r, st.beta, st.active, nrhs, par0, npar, s);
 }
 

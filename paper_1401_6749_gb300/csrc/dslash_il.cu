@@ -79,8 +79,6 @@ struct IlArgs {
   const uint2* in;
   uint2* out;
   const uint2* cfield;    // centre field (null: in)
-  const uint2* p;
-  uint2* x;
   uint2* r;
   const uint2* b;
   const int* active;
@@ -213,7 +211,7 @@ struct IlStage {
 // partial sums (the CG update and the residual always do)
 constexpr int kIlNorm = 8;
 template <class S, bool DAG, int EPI, int FORM>
-__global__ void __launch_bounds__(kIlWarps * 32, EPI == EPI_CGUPD ? 3 : 4)
+__global__ void __launch_bounds__(kIlWarps * 32, 4)
     dslash_il_kernel(const IlArgs a, const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tlk) {
   using H = H16<S>;
   constexpr int CENTRE = (FORM & 7) >> 1;
@@ -319,7 +317,6 @@ __global__ void __launch_bounds__(kIlWarps * 32, EPI == EPI_CGUPD ? 3 : 4)
       al0 = act0 ? (float)a.alpha[r0] : 0.0f;
       al1 = act1 ? (float)a.alpha[r1] : 0.0f;
     }
-    const float2 pal0 = make_float2(al0, al0), pal1 = make_float2(al1, al1);
     const float2 nal0 = make_float2(-al0, -al0), nal1 = make_float2(-al1, -al1);
     unsigned char* ring = il_smem + wq * ST::kWarpBytes;
     const unsigned ring_s = smem_u32(ring);
@@ -335,23 +332,14 @@ __global__ void __launch_bounds__(kIlWarps * 32, EPI == EPI_CGUPD ? 3 : 4)
     const size_t lbase = (obase + woff) / 8;
     const uint2* cf = (a.cfield ? a.cfield : a.in) + lbase;
     const uint2* rp = (EPI == EPI_RESID ? a.b : a.r) + lbase;
-    const uint2* xp = a.x + lbase;
-    const uint2* pp = a.p + lbase;
     uint2* op = (EPI == EPI_CGUPD ? a.r : a.out) + lbase;
-    uint2* oxp = a.x + lbase;
-    uint2 cw[4], rw[4], xw[4], pw[4];
+    uint2 cw[4], rw[4];
     auto fetch_site = [&](int m) {
       const unsigned w = (unsigned)(base + wq + kIlWarps * m) * (kIlSiteBytes / 8);
 #pragma unroll
       for (int s = 0; s < 4; ++s) {
         if constexpr (CENTRE != 0) cw[s] = cf[w + 24 * s];
-        if constexpr (EPI == EPI_CGUPD) {
-          rw[s] = rp[w + 24 * s];
-          xw[s] = xp[w + 24 * s];
-          pw[s] = pp[w + 24 * s];
-        } else if constexpr (EPI == EPI_RESID) {
-          rw[s] = rp[w + 24 * s];
-        }
+        if constexpr (EPI != EPI_OUT) rw[s] = rp[w + 24 * s];
       }
     };
     // returns the site's wrap mask (the next iteration's time-boundary signs)
@@ -420,7 +408,6 @@ __global__ void __launch_bounds__(kIlWarps * 32, EPI == EPI_CGUPD ? 3 : 4)
       // epilogue: out = T_out(T_c(c) + s_hop H in), then the CG update / residual;
       // lanes t = 3 compute on the words of t = 0 and store nothing
       uint2* const ost = op + (unsigned)(base + wq + kIlWarps * m) * (kIlSiteBytes / 8);
-      uint2* const xst = oxp + (unsigned)(base + wq + kIlWarps * m) * (kIlSiteBytes / 8);
       // the hopping sum of each spin (rows g, g + 8: re, im, re, im)
       float hs[4][4];
 #pragma unroll
@@ -473,20 +460,14 @@ __global__ void __launch_bounds__(kIlWarps * 32, EPI == EPI_CGUPD ? 3 : 4)
             n1 = __ffma2_rn(o1, o1, n1);
           }
         } else if constexpr (EPI == EPI_CGUPD) {
-          // r and x of inactive systems keep their bits
+          // r of inactive systems keeps its bits (x follows in the xpay pass)
           float2 q0 = H::to_f2(rw[s].x), q1 = H::to_f2(rw[s].y);
           q0 = __ffma2_rn(nal0, o0, q0);
           q1 = __ffma2_rn(nal1, o1, q1);
           const uint2 rn = make_uint2(act0 ? H::pack(q0.x, q0.y) : rw[s].x, act1 ? H::pack(q1.x, q1.y) : rw[s].y);
           n0 = __ffma2_rn(q0, q0, n0);
           n1 = __ffma2_rn(q1, q1, n1);
-          const float2 x0 = __ffma2_rn(pal0, H::to_f2(pw[s].x), H::to_f2(xw[s].x));
-          const float2 x1 = __ffma2_rn(pal1, H::to_f2(pw[s].y), H::to_f2(xw[s].y));
-          const uint2 xn = make_uint2(act0 ? H::pack(x0.x, x0.y) : xw[s].x, act1 ? H::pack(x1.x, x1.y) : xw[s].y);
-          if (l.ld) {
-            ost[24 * s] = rn;
-            xst[24 * s] = xn;
-          }
+          if (l.ld) ost[24 * s] = rn;
         } else {  // EPI_RESID: out = b - D in
           const float2 m1 = make_float2(-1.0f, -1.0f);  // b - o, rounded once as by a subtraction
           o0 = __ffma2_rn(m1, o0, H::to_f2(rw[s].x));
@@ -622,8 +603,6 @@ static tm_status_t il_launch_t(const tm_op* op, const DslashCall& c, cudaStream_
   a.in = static_cast<const uint2*>(c.in);
   a.out = static_cast<uint2*>(c.out);
   a.cfield = static_cast<const uint2*>(c.cfield);
-  a.p = static_cast<const uint2*>(c.p);
-  a.x = static_cast<uint2*>(c.x);
   a.r = static_cast<uint2*>(c.r);
   a.b = static_cast<const uint2*>(c.b);
   a.active = c.active;
@@ -651,7 +630,7 @@ static tm_status_t il_launch_t(const tm_op* op, const DslashCall& c, cudaStream_
   a.inv = (float)(1.0 / (1.0 + nu * nu));
   a.sinv = (float)(hop / (1.0 + nu * nu));
   // every field the bulk copies read must sit on a 16-byte boundary
-  const void* ptrs[6] = {a.in, a.cfield, a.p, a.x, a.r, a.b};
+  const void* ptrs[4] = {a.in, a.cfield, a.r, a.b};
   for (const void* q : ptrs)
     if (q && ((uintptr_t)q & 15u)) {
       set_error("dslash_il: fields must be 16-byte aligned");
@@ -686,11 +665,11 @@ static tm_status_t il_launch_t(const tm_op* op, const DslashCall& c, cudaStream_
   const double out_sites = (double)npar * g.Vh;
   const bool centre_is_in = a.cfield == nullptr || a.cfield == a.in;
   const int centre = (a.centre != 0 && !(c.parity < 0 && centre_is_in)) ? 1 : 0;
-  const int epi_streams = EPI == EPI_OUT ? 1 : (EPI == EPI_CGUPD ? 5 : 2);
+  const int epi_streams = EPI == EPI_OUT ? 1 : 2;
   const double per_rhs = out_sites * 24.0 * e * (1 + centre + epi_streams);
   const double fixed = 4.0 * 2.0 * g.Vh * 18.0 * e;
   const double site_flops = 1320.0 + 48.0 + (a.centre == 2 ? 48.0 : 0.0) + (a.out_inv ? 72.0 : 0.0) +
-                            (EPI == EPI_CGUPD ? 144.0 : EPI == EPI_RESID ? 72.0 : (a.partial ? 48.0 : 0.0));
+                            (EPI == EPI_CGUPD ? 96.0 : EPI == EPI_RESID ? 72.0 : (a.partial ? 48.0 : 0.0));
   const int form = 2 * a.centre + a.out_inv;
   if (EPI != EPI_OUT && form != 4) {
     set_error("dslash_il: the CG update and residual forms need the twisted centre without A^-1");
@@ -877,15 +856,18 @@ tm_status_t il_convert(const Geom& g, void* out, const void* in, int nrhs, bool 
 }
 
 // ------------------------------------------------ solver BLAS on IL16
-// p = r + beta p for the active systems on parities par0 .. par0 + npar - 1.
+// The vector updates of a CG iteration on parities par0 .. par0 + npar - 1: x += alpha p
+// for the systems that took the step (alpha != 0), then p = r + beta p for the
+// active ones.  x moves with p here and not in the Dslash's update of r, so that
+// p is read once: five streams here and four there instead of three and seven.
 // One plane (block of systems, parity) per grid row; a thread takes 16-byte
-// words (pair positions 2q, 2q + 1 of a row), the systems' beta and flags
-// come from shared memory.
+// words (pair positions 2q, 2q + 1 of a row), the systems' scalars come from
+// shared memory.
 template <class S>
-__global__ void il_xpay_kernel(uint4* p, const uint4* r, const double* beta, const int* active, int nrhs,
-                               int par0, int npar, unsigned plane_u4) {
+__global__ void il_xpay_kernel(uint4* x, uint4* p, const uint4* r, const double* alpha, const double* beta,
+                               const int* active, int nrhs, int par0, int npar, unsigned plane_u4) {
   using H = H16<S>;
-  __shared__ float sb[kIlRows];
+  __shared__ float sb[kIlRows], sl[kIlRows];
   __shared__ int sa[kIlRows];
   const int blk = blockIdx.y / npar, pi = blockIdx.y % npar;
   if (threadIdx.x < kIlRows) {
@@ -893,75 +875,85 @@ __global__ void il_xpay_kernel(uint4* p, const uint4* r, const double* beta, con
     const int on = rr < nrhs && active[rr] != 0;
     sa[threadIdx.x] = on;
     sb[threadIdx.x] = on ? (float)beta[rr] : 0.0f;
+    sl[threadIdx.x] = rr < nrhs ? (float)alpha[rr] : 0.0f;
   }
   __syncthreads();
-  uint4* pp = p + ((size_t)blk * 2 + par0 + pi) * plane_u4;
-  const uint4* rp = r + ((size_t)blk * 2 + par0 + pi) * plane_u4;
+  const size_t off = ((size_t)blk * 2 + par0 + pi) * plane_u4;
+  uint4* xp = x + off;
+  uint4* pp = p + off;
+  const uint4* rp = r + off;
   for (unsigned j = blockIdx.x * blockDim.x + threadIdx.x; j < plane_u4; j += gridDim.x * blockDim.x) {
     const unsigned k = (j >> 2) % 12u;  // row j / 4 = site * 12 + k
     const int sw = k % 3u == 2u ? 4 : 0;
     const int g0 = (int)(2 * (j & 3)) ^ sw, g1 = (int)(2 * (j & 3) + 1) ^ sw;
+    const float l0 = sl[g0], l1 = sl[g0 + 8], l2 = sl[g1], l3 = sl[g1 + 8];
+    if (l0 == 0.0f && l1 == 0.0f && l2 == 0.0f && l3 == 0.0f) continue;  // an active system has taken a step
     const bool a0 = sa[g0], a1 = sa[g0 + 8], a2 = sa[g1], a3 = sa[g1 + 8];
-    if (!(a0 || a1 || a2 || a3)) continue;
     const float b0 = sb[g0], b1 = sb[g0 + 8], b2 = sb[g1], b3 = sb[g1 + 8];
-    const uint4 rv = rp[j], pv = pp[j];
-    auto upd = [&](unsigned rw, unsigned pw, float b, bool on) -> unsigned {
-      const float2 x = H::to_f2(rw), y = H::to_f2(pw);
-      return on ? H::pack(__fmaf_rn(b, y.x, x.x), __fmaf_rn(b, y.y, x.y)) : pw;
+    const uint4 rv = rp[j], pv = pp[j], xv = xp[j];
+    auto step = [&](unsigned xw, unsigned pw, float l) -> unsigned {
+      const float2 u = H::to_f2(xw), y = H::to_f2(pw);
+      return l != 0.0f ? H::pack(__fmaf_rn(l, y.x, u.x), __fmaf_rn(l, y.y, u.y)) : xw;
     };
-    pp[j] = make_uint4(upd(rv.x, pv.x, b0, a0), upd(rv.y, pv.y, b1, a1), upd(rv.z, pv.z, b2, a2),
-                       upd(rv.w, pv.w, b3, a3));
+    auto upd = [&](unsigned rw, unsigned pw, float b, bool on) -> unsigned {
+      const float2 u = H::to_f2(rw), y = H::to_f2(pw);
+      return on ? H::pack(__fmaf_rn(b, y.x, u.x), __fmaf_rn(b, y.y, u.y)) : pw;
+    };
+    xp[j] = make_uint4(step(xv.x, pv.x, l0), step(xv.y, pv.y, l1), step(xv.z, pv.z, l2), step(xv.w, pv.w, l3));
+    if (a0 || a1 || a2 || a3)
+      pp[j] = make_uint4(upd(rv.x, pv.x, b0, a0), upd(rv.y, pv.y, b1, a1), upd(rv.z, pv.z, b2, a2),
+                         upd(rv.w, pv.w, b3, a3));
   }
 }
 
-tm_status_t il_xpay(const Geom& g, tm_prec_t prec, void* p, const void* r, const double* beta,
-                    const int* active, int nrhs, int par0, int npar, cudaStream_t s) {
+tm_status_t il_xpay(const Geom& g, tm_prec_t prec, void* x, void* p, const void* r, const double* alpha,
+                    const double* beta, const int* active, int nrhs, int par0, int npar, cudaStream_t s) {
   const int nblk = (nrhs + kIlRows - 1) / kIlRows;
   const unsigned plane_u4 = (unsigned)((size_t)g.Vh * (kIlSiteBytes / 16));
   const unsigned gx = std::min<unsigned>((plane_u4 + 255) / 256, 152u * 8u);
   const dim3 grid(gx, (unsigned)(nblk * npar));
-  TraceScope tr(s, "blas.xpay", 3.0 * 24.0 * 2.0 * npar * g.Vh, 0.0, nrhs);
+  TraceScope tr(s, "blas.xpay", 5.0 * 24.0 * 2.0 * npar * g.Vh, 0.0, nrhs);
   if (prec == TM_PREC_F16)
-    il_xpay_kernel<__half><<<grid, 256, 0, s>>>(static_cast<uint4*>(p), static_cast<const uint4*>(r), beta, active,
-                                                nrhs, par0, npar, plane_u4);
+    il_xpay_kernel<__half><<<grid, 256, 0, s>>>(static_cast<uint4*>(x), static_cast<uint4*>(p),
+                                                static_cast<const uint4*>(r), alpha, beta, active, nrhs, par0, npar,
+                                                plane_u4);
   else
-    il_xpay_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(static_cast<uint4*>(p), static_cast<const uint4*>(r), beta,
-                                                       active, nrhs, par0, npar, plane_u4);
+    il_xpay_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(static_cast<uint4*>(x), static_cast<uint4*>(p),
+                                                       static_cast<const uint4*>(r), alpha, beta, active, nrhs, par0,
+                                                       npar, plane_u4);
   count_launch();
   return check_launch("xpay (interleaved)");
 }
 
 // out = A in (inverse = 0) or A^-1 in (inverse = 1) on one parity, as twist()
 template <class S>
-__global__ void il_twist_kernel(size_t Vh, uint2* out, const uint2* in, float tn, float sc, int nblk, int par) {
+__global__ void __launch_bounds__(256) il_twist_kernel(unsigned per_blk, uint4* out, const uint4* in, float tn,
+                                                       float sc, int par) {
   using H = H16<S>;
-  const size_t per_blk = Vh * kIlSiteU2;
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= per_blk * nblk) return;
-  const int blk = (int)(i / per_blk);
-  const size_t rem = i % per_blk;
-  const int k = (int)((rem >> 3) % 12);
-  const size_t w = ((size_t)blk * 2 + par) * per_blk + rem;
-  const float tw = k < 6 ? tn : -tn;
-  const uint2 v = in[w];
-  const float2 c0 = H::to_f2(v.x), c1 = H::to_f2(v.y);
-  out[w] = make_uint2(H::pack(__fmul_rn(sc, __fmaf_rn(-tw, c0.y, c0.x)), __fmul_rn(sc, __fmaf_rn(tw, c0.x, c0.y))),
-                      H::pack(__fmul_rn(sc, __fmaf_rn(-tw, c1.y, c1.x)), __fmul_rn(sc, __fmaf_rn(tw, c1.x, c1.y))));
+  const unsigned rem = blockIdx.x * blockDim.x + threadIdx.x;  // 16-byte word of the plane
+  if (rem >= per_blk) return;
+  const size_t w = ((size_t)blockIdx.y * 2 + par) * per_blk + rem;
+  const float tw = (rem >> 2) % 12u < 6u ? tn : -tn;
+  const uint4 v = in[w];
+  auto f = [&](unsigned q) {
+    const float2 c = H::to_f2(q);
+    return H::pack(__fmul_rn(sc, __fmaf_rn(-tw, c.y, c.x)), __fmul_rn(sc, __fmaf_rn(tw, c.x, c.y)));
+  };
+  out[w] = make_uint4(f(v.x), f(v.y), f(v.z), f(v.w));
 }
 
 tm_status_t il_twist(const Geom& g, tm_prec_t prec, void* out, const void* in, double nu, int inverse, int par,
                      int nrhs, cudaStream_t s) {
   const int nblk = (nrhs + kIlRows - 1) / kIlRows;
-  const size_t n = (size_t)nblk * (size_t)g.Vh * kIlSiteU2;
-  const unsigned nb = (unsigned)((n + 255) / 256);
+  const unsigned n = (unsigned)((size_t)g.Vh * (kIlSiteBytes / 16));
+  const dim3 grid((n + 255) / 256, (unsigned)nblk);
   const float sc = inverse ? (float)(1.0 / (1.0 + nu * nu)) : 1.0f;
   const float tn = inverse ? (float)(-nu) : (float)nu;
   if (prec == TM_PREC_F16)
-    il_twist_kernel<__half><<<nb, 256, 0, s>>>((size_t)g.Vh, static_cast<uint2*>(out),
-                                                static_cast<const uint2*>(in), tn, sc, nblk, par);
+    il_twist_kernel<__half><<<grid, 256, 0, s>>>(n, static_cast<uint4*>(out), static_cast<const uint4*>(in), tn, sc, par);
   else
-    il_twist_kernel<__nv_bfloat16><<<nb, 256, 0, s>>>((size_t)g.Vh, static_cast<uint2*>(out),
-                                                       static_cast<const uint2*>(in), tn, sc, nblk, par);
+    il_twist_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(n, static_cast<uint4*>(out), static_cast<const uint4*>(in), tn,
+                                                        sc, par);
   count_launch();
   return check_launch("twist (interleaved)");
 }

@@ -95,6 +95,7 @@ enum Epi { EPI_OUT = 0, EPI_CGUPD = 1, EPI_RESID = 2 };
 // One Dslash application over nrhs fields, with an optional fused epilogue.
 //   EPI_OUT   : out = D in;                 partial |out|^2 if partial != null
 //   EPI_CGUPD : q = D in (not stored); r -= alpha q; x += alpha p;  partial |r|^2
+//               (interleaved layout: x follows in il_xpay, p and x unused)
 //   EPI_RESID : out = b - D in;             partial |out|^2
 // D = M, M^dag (dagger) or D_W (mu_zero).  Systems with active[rhs] == 0
 // are skipped entirely (no stores, zero partial).  Partial sums are written
@@ -144,8 +145,8 @@ tm_status_t dslash_dispatch(const tm_op* op, tm_prec_t prec, const DslashCall& c
 size_t il_bytes(const Geom& g, int nrhs);
 tm_status_t dslash_il_dispatch(const tm_op* op, tm_prec_t prec, const DslashCall& c, cudaStream_t s);
 tm_status_t il_convert(const Geom& g, void* out, const void* in, int nrhs, bool to_il, cudaStream_t s);
-tm_status_t il_xpay(const Geom& g, tm_prec_t prec, void* p, const void* r, const double* beta,
-                    const int* active, int nrhs, int par0, int npar, cudaStream_t s);
+tm_status_t il_xpay(const Geom& g, tm_prec_t prec, void* x, void* p, const void* r, const double* alpha,
+                    const double* beta, const int* active, int nrhs, int par0, int npar, cudaStream_t s);
 tm_status_t il_twist(const Geom& g, tm_prec_t prec, void* out, const void* in, double nu, int inverse, int par,
                      int nrhs, cudaStream_t s);
 bool cg_il_on();
