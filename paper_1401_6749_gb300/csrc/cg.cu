@@ -7,10 +7,10 @@
 //
 // Per iteration (PLAIN, every vector in one precision):
 //   t = M p                       Dslash, fused |t|^2 per-warp partials
-//   alpha = |r|^2 / |t|^2         fixed-order reduction + scalar kernel
+//   alpha = |r|^2 / |t|^2         fixed-order reduction and scalar step, one kernel
 //   r -= alpha M^dag t, x += alpha p   Dslash with fused update, |r|^2 partials (on
 //                                  the interleaved layout x moves with p below)
-//   beta = |r_new|^2 / |r|^2      fixed-order reduction + scalar kernel
+//   beta = |r_new|^2 / |r|^2      fixed-order reduction and scalar step, one kernel
 //   p = r + beta p
 // MIXED adds FP64 reliable updates (Sleijpen & van der Vorst): the iteration
 // runs in inner precision on a correction y; when |r| drops below delta times
@@ -141,13 +141,15 @@ struct CgScalars {
   int mixed;
 };
 
-__global__ void cg_init_kernel(CgState st, CgScalars sc) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= sc.nrhs) return;
+// scale of the inner vectors for a mean square m of the residual's entries: the
+// power of two at or below its root, so that scaling by it is exact
+__device__ __forceinline__ double cg_sigma(double m) { return scalbn(1.0, ilogb(sqrt(m))); }
+
+__device__ __forceinline__ void cg_init(const CgState& st, const CgScalars& sc, int i) {
   const double bb = st.red[i];
   // MIXED: the inner iteration runs on b / sigma with entries of order one,
   // so that narrow formats (FP16) neither overflow nor underflow
-  const double sg = (sc.mixed && bb > 0.0 && isfinite(bb)) ? sqrt(bb / sc.n12) : 1.0;
+  const double sg = (sc.mixed && bb > 0.0 && isfinite(bb)) ? cg_sigma(bb / sc.n12) : 1.0;
   st.bb[i] = bb;
   st.sigma[i] = sg;
   st.ratio[i] = 1.0;
@@ -168,9 +170,7 @@ __global__ void cg_init_kernel(CgState st, CgScalars sc) {
   }
 }
 
-__global__ void cg_alpha_kernel(CgState st, CgScalars sc) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= sc.nrhs) return;
+__device__ __forceinline__ void cg_alpha(const CgState& st, const CgScalars& sc, int i) {
   st.ru[i] = 0;  // the reliable update of the previous iteration is complete
   if (!st.active[i]) {
     st.alpha[i] = 0.0;  // no step: il_xpay leaves x alone
@@ -186,9 +186,8 @@ __global__ void cg_alpha_kernel(CgState st, CgScalars sc) {
   st.alpha[i] = st.rr[i] / pap;
 }
 
-__global__ void cg_beta_plain_kernel(CgState st, CgScalars sc) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= sc.nrhs || !st.active[i]) return;
+__device__ __forceinline__ void cg_beta_plain(const CgState& st, const CgScalars& sc, int i) {
+  if (!st.active[i]) return;
   const double rn = st.red[i];
   const int it = ++st.iters[i];
   if (!isfinite(rn)) {
@@ -207,9 +206,8 @@ __global__ void cg_beta_plain_kernel(CgState st, CgScalars sc) {
   }
 }
 
-__global__ void cg_beta_mixed_kernel(CgState st, CgScalars sc) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= sc.nrhs || !st.active[i]) return;
+__device__ __forceinline__ void cg_beta_mixed(const CgState& st, const CgScalars& sc, int i) {
+  if (!st.active[i]) return;
   const double rn = st.red[i];
   const int it = ++st.iters[i];
   if (!isfinite(rn)) {
@@ -227,9 +225,8 @@ __global__ void cg_beta_mixed_kernel(CgState st, CgScalars sc) {
   st.rr[i] = rn;
 }
 
-__global__ void cg_ru_kernel(CgState st, CgScalars sc) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= sc.nrhs || !st.ru[i]) return;
+__device__ __forceinline__ void cg_ru(const CgState& st, const CgScalars& sc, int i) {
+  if (!st.ru[i]) return;
   const double rt = st.red[i];  // |b - M^dag M x|^2, absolute
   st.nru[i] += 1;
   if (!isfinite(rt)) {
@@ -239,7 +236,7 @@ __global__ void cg_ru_kernel(CgState st, CgScalars sc) {
     return;
   }
   const double s_old = st.sigma[i];
-  const double s_new = rt > 0.0 ? sqrt(rt / sc.n12) : s_old;
+  const double s_new = rt > 0.0 ? cg_sigma(rt / sc.n12) : s_old;
   st.beta[i] = rt / (st.rr[i] * s_old * s_old);
   st.rr[i] = rt / (s_new * s_new);
   st.sigma[i] = s_new;
@@ -252,6 +249,26 @@ __global__ void cg_ru_kernel(CgState st, CgScalars sc) {
     st.active[i] = 0;
     st.status[i] = TM_ERR_NOCONV;
   }
+}
+
+// A reduction and the scalar step that follows from it, one block per system:
+// red = the system's partial sums in the fixed order of reduce_partials, then the
+// step of its scalars (one launch instead of two: at 4^4 an iteration is seven
+// launches of 2 to 17 us)
+enum CgStep { CG_INIT, CG_ALPHA, CG_BETA_PLAIN, CG_BETA_MIXED, CG_RU };
+
+template <CgStep STEP>
+__global__ void __launch_bounds__(256) cg_step_kernel(const double* partial, int nper, size_t stride, CgState st,
+                                                      CgScalars sc) {
+  const int i = blockIdx.x;
+  const double v = block_sum(partial + (size_t)i * stride, nper);
+  if (threadIdx.x != 0) return;
+  st.red[i] = v;
+  if constexpr (STEP == CG_INIT) cg_init(st, sc, i);
+  else if constexpr (STEP == CG_ALPHA) cg_alpha(st, sc, i);
+  else if constexpr (STEP == CG_BETA_PLAIN) cg_beta_plain(st, sc, i);
+  else if constexpr (STEP == CG_BETA_MIXED) cg_beta_mixed(st, sc, i);
+  else cg_ru(st, sc, i);
 }
 
 static size_t align_up(size_t n) { return (n + 255) & ~(size_t)255; }
@@ -292,14 +309,6 @@ static tm_status_t ensure_work(tm_op* op, size_t bytes, int nflags, cudaStream_t
     }
   }
   return TM_OK;
-}
-
-static tm_status_t scalar_launch(void (*k)(CgState, CgScalars), const CgState& st,
-                                 const CgScalars& sc, cudaStream_t s) {
-  const int nb = (sc.nrhs + 127) / 128;
-  k<<<nb, 128, 0, s>>>(st, sc);
-  count_launch();
-  return check_launch("cg scalar kernel");
 }
 
 // The planes of parities par0 .. par0 + npar - 1 of `rows` fields (or blocks of
@@ -375,6 +384,13 @@ struct CgRun {
 
   SolveOp A() const { return SolveOp{op, schur, nrhs, s, il}; }
   tm_status_t reduce() const { return reduce_partials(part0, nper, nrhs, st.red, s, pstride); }
+  // reduction of the partial sums and the scalar step that uses it
+  template <CgStep STEP>
+  tm_status_t step() const {
+    cg_step_kernel<STEP><<<nrhs, 256, 0, s>>>(part0, nper, pstride, st, sc);
+    count_launch();
+    return check_launch("cg step");
+  }
 
   tm_status_t setup();
   tm_status_t iteration();
@@ -489,8 +505,7 @@ tm_status_t CgRun::setup() {
       e.il = il;
       TM_TRY(dslash_dispatch(op, hi, e, s));
     }
-    TM_TRY(reduce());
-    TM_TRY(scalar_launch(cg_init_kernel, st, sc, s));
+    TM_TRY(step<CG_INIT>());
   }
   // vectors are initialised on the parities they live on (the other half of a
   // Schur solve's is scratch)
@@ -518,17 +533,15 @@ tm_status_t CgRun::iteration() {
   const Geom& g = op->g;
   const SolveOp Op = A();
   TM_TRY(Op.apply(lo, p, t, partial, st.active));  // t = Op p, |t|^2
-  TM_TRY(reduce());
-  TM_TRY(scalar_launch(cg_alpha_kernel, st, sc, s));
+  TM_TRY(step<CG_ALPHA>());
   DslashCall e;  // r -= alpha Op^dag t, x += alpha p, |r|^2
   e.epi = EPI_CGUPD; e.partial = partial; e.active = st.active; e.alpha = st.alpha;
   e.p = p; e.x = xs; e.r = r;
   TM_TRY(Op.apply_dag(lo, t, e));
-  TM_TRY(reduce());
   if (!mixed) {
-    TM_TRY(scalar_launch(cg_beta_plain_kernel, st, sc, s));
+    TM_TRY(step<CG_BETA_PLAIN>());
   } else {
-    TM_TRY(scalar_launch(cg_beta_mixed_kernel, st, sc, s));
+    TM_TRY(step<CG_BETA_MIXED>());
     // reliable update for the systems that asked for one: x += sigma y (FP64),
     // r = b - Op^dag Op x in FP64 or float-float (ru_prec)
     TM_TRY(fold(g, lo, x, y, st.sigma, st.ru, nrhs, par0, npar, s, ru_ff ? xff : nullptr));
@@ -536,8 +549,7 @@ tm_status_t CgRun::iteration() {
     DslashCall e4;
     e4.out = r64; e4.b = ru_ff ? bff : b64; e4.epi = EPI_RESID; e4.partial = partial; e4.active = st.ru;
     TM_TRY(Op.apply_dag(ru, tmp64, e4));
-    TM_TRY(reduce());
-    TM_TRY(scalar_launch(cg_ru_kernel, st, sc, s));
+    TM_TRY(step<CG_RU>());
     TM_TRY(rescale(g, lo, r, r64, st.sigma, p, st.ratio, st.ru, nrhs, par0, npar, s, ru_ff));
   }
   if (il) return il_xpay(g, lo, xs, p, r, st.alpha, st.beta, st.active, nrhs, par0, npar, s);

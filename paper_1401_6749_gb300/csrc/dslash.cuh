@@ -771,14 +771,17 @@ tm_status_t launch_one(const tm_op* op, const DslashCall& c, cudaStream_t st, in
     }
   }
   int lgs = 0;
+  bool quad = false;
   if constexpr (HALF) {
     // pairs of warps, two to a block; where there are too few for every SM,
-    // one to a block
+    // four warps per 32 sites (FP64) or one pair to a block
     const long pairs = (long)a.nwarp * (c.parity < 0 ? 2 : 1) * c.nrhs;
-    bx = pairs < 2 * 152 ? 64 : 128;
-    lgs = bx == 128 && c.nrhs >= 2 ? 1 : 0;
+    const bool few = pairs < 2 * 152;
+    quad = few && std::is_same<S, double>::value;
+    bx = few && !quad ? 64 : 128;
+    lgs = !few && c.nrhs >= 2 ? 1 : 0;
     a.rhs_groups = (c.nrhs + (1 << lgs) - 1) >> lgs;
-    const int gpb = bx >> (6 + lgs);  // 32-site groups per block
+    const int gpb = quad ? 1 : bx >> (6 + lgs);  // 32-site groups per block
     const int gb = (a.nwarp + gpb - 1) / gpb;
     grid = dim3((unsigned)((c.parity < 0 ? 2 * gb : gb) * a.rhs_groups));
   }
@@ -806,9 +809,11 @@ tm_status_t launch_one(const tm_op* op, const DslashCall& c, cudaStream_t st, in
   const double fixed = 4.0 * 2.0 * op->g.Vh * link_reals * e;
   cudaEvent_t ev = nullptr;
   a.trace_count = trace_begin(st, &ev);
-  if constexpr (HALF && std::is_same<S, double>::value)
-    dslash_fx_kernel<DAG, EPI><<<grid, bx, 0, st>>>(a, static_cast<const int4*>(op->links_fx), lgs);
-  else if constexpr (HALF) dslash_ff_kernel<DAG, EPI><<<grid, bx, 0, st>>>(a, lgs);
+  if constexpr (HALF && std::is_same<S, double>::value) {
+    const int4* lf = static_cast<const int4*>(op->links_fx);
+    if (quad) dslash_fx_kernel<DAG, EPI, true><<<grid, bx, 0, st>>>(a, lf, lgs);
+    else dslash_fx_kernel<DAG, EPI, false><<<grid, bx, 0, st>>>(a, lf, lgs);
+  } else if constexpr (HALF) dslash_ff_kernel<DAG, EPI><<<grid, bx, 0, st>>>(a, lgs);
   else if constexpr (MMA) dslash_kernel_mma<S, DAG, EPI><<<grid, kMmaThreads, kMmaSmem, st>>>(a);
   else if constexpr (X2) dslash_kernel_x2<S, RECON, DAG, EPI><<<grid, bx, 0, st>>>(a);
   else dslash_kernel<S, RECON, DAG, EPI, NR><<<grid, bx, 0, st>>>(a);

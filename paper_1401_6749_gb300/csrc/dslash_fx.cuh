@@ -198,19 +198,19 @@ __device__ __noinline__ void hop_sum_f64(Cx<double>* out, const Geom* gp, const 
   for (int k = 0; k < 12; ++k) out[k] = acc[k];
 }
 
-// The FP64 epilogue (dslash_epilogue) of the components of spins sp and 2 + sp:
-// acc[0..2] and acc[3..5] the hopping sums in units of `unit`.  Returns their
-// |.|^2.
-template <int EPI, int CENTRE, bool INV>
-__device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp, int r, int par, int cb, double unit,
-                                              const Cx<double> (&acc)[6]) {
+// The FP64 epilogue (dslash_epilogue) of spin sp0 (acc[0..2]) and, with NC = 6,
+// spin sp0 + 2 (acc[3..5]); acc the hopping sums in units of `unit`.  Returns
+// their |.|^2.
+template <int EPI, int CENTRE, bool INV, int NC>
+__device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp0, int r, int par, int cb, double unit,
+                                              const Cx<double> (&acc)[NC]) {
   const size_t cs = (size_t)a.g.Vh;
-  const size_t b0 = ((size_t)(r * 2 + par) * 12 + 3 * sp) * cs + cb;  // chunk q: + (q < 3 ? q : q + 3) cs
-  const double nu = a.nu, inv = a.inv;
+  const size_t b0 = ((size_t)(r * 2 + par) * 12 + 3 * sp0) * cs + cb;  // chunk q: + (q < 3 ? q : q + 3) cs
+  const double nu = sp0 < 2 ? a.nu : -a.nu, inv = a.inv;
   const double shop = CENTRE == 0 && INV ? a.hop_scale * unit * inv : a.hop_scale * unit;
-  Cx<double> o[6];
+  Cx<double> o[NC];
 #pragma unroll
-  for (int q = 0; q < 6; ++q) {
+  for (int q = 0; q < NC; ++q) {
     const double tw = q < 3 ? nu : -nu;  // gamma_5 = diag(1, 1, -1, -1)
     const Cx<double> v = acc[q];
     if constexpr (CENTRE != 0) {
@@ -229,13 +229,13 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp, int r
   if constexpr (EPI == EPI_OUT) {
     double2* out = reinterpret_cast<double2*>(a.c.out) + b0;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      if (q >= 3 && a.c.g5_out) o[q] = {-o[q].re, -o[q].im};
+    for (int q = 0; q < NC; ++q) {
+      if ((q >= 3 || sp0 >= 2) && a.c.g5_out) o[q] = {-o[q].re, -o[q].im};
       out[(q < 3 ? q : q + 3) * cs] = make_double2(o[q].re, o[q].im);
     }
     if (a.c.partial) {
 #pragma unroll
-      for (int q = 0; q < 6; ++q) part = __fma_rn(o[q].re, o[q].re, __fma_rn(o[q].im, o[q].im, part));
+      for (int q = 0; q < NC; ++q) part = __fma_rn(o[q].re, o[q].re, __fma_rn(o[q].im, o[q].im, part));
     }
   } else if constexpr (EPI == EPI_CGUPD) {
     const double al = a.c.alpha[r];
@@ -243,7 +243,7 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp, int r
     double2* xf = reinterpret_cast<double2*>(a.c.x) + b0;
     const double2* pf = reinterpret_cast<const double2*>(a.c.p) + b0;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
+    for (int q = 0; q < NC; ++q) {
       const size_t i = (q < 3 ? q : q + 3) * cs;
       const double2 v = rf[i], x = xf[i], p = pf[i];
       const double2 n = make_double2(__fma_rn(-al, o[q].re, v.x), __fma_rn(-al, o[q].im, v.y));
@@ -255,7 +255,7 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp, int r
     const double2* bf = reinterpret_cast<const double2*>(a.c.b) + b0;
     double2* out = reinterpret_cast<double2*>(a.c.out) + b0;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
+    for (int q = 0; q < NC; ++q) {
       const size_t i = (q < 3 ? q : q + 3) * cs;
       const double2 v = bf[i];
       const double2 n = make_double2(__dsub_rn(v.x, o[q].re), __dsub_rn(v.y, o[q].im));
@@ -277,7 +277,7 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp, int r
 // 36.6 us (there one block's chain of instructions).  Measured beside it: one
 // thread per site unrolled over the hops, 2.43 ms and 21.7 us; the input
 // converted once by a pass of its own, 2.19 ms with the pass, 22 us.
-template <bool DAG, int EPI>
+template <bool DAG, int EPI, bool QUAD>
 __global__ void __launch_bounds__(128, 4) dslash_fx_kernel(const DslashArgs a, const int4* links_fx, int lgs) {
   __shared__ longlong2 xch[4][3][32];
   __shared__ unsigned xe[4][32][2];
@@ -288,8 +288,9 @@ __global__ void __launch_bounds__(128, 4) dslash_fx_kernel(const DslashArgs a, c
   const int par = a.c.parity < 0 ? (sb & 1) : a.c.parity;
   const int gb = a.c.parity < 0 ? (sb >> 1) : sb;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int sp = warp & 1, pair = warp >> 1;
-  const int grp = gb * (int)(blockDim.x >> (6 + lgs)) + (pair >> lgs);  // 32-site group
+  const int sp = warp & 1, pair = QUAD ? 0 : warp >> 1;
+  const int it0 = QUAD ? warp >> 1 : 0, it1 = QUAD ? it0 + 1 : 2;  // pairs of directions of this warp
+  const int grp = QUAD ? gb : gb * (int)(blockDim.x >> (6 + lgs)) + (pair >> lgs);  // 32-site group
   const int cb = grp * 32 + lane;
   const int r = (rg << lgs) + (pair & ((1 << lgs) - 1));
   const int nrhs = a.c.nrhs;
@@ -311,7 +312,7 @@ __global__ void __launch_bounds__(128, 4) dslash_fx_kernel(const DslashArgs a, c
 #pragma unroll
     for (int c = 0; c < 3; ++c) t.upr[c] = t.upi[c] = 0;
 #pragma unroll 1
-    for (int it = 0; it < 2; ++it) {
+    for (int it = it0; it < it1; ++it) {
       const int4* uf = links_fx + (size_t)(4 * it + par) * a.nwarp * 288;  // direction 2 it; the next one: + 576 nwarp
       const int4* ub = links_fx + (size_t)(4 * it + opar) * a.nwarp * 288;
       const double2* fdn = fup + (6 + 3 * (it ? 0 : 1 - 2 * sp)) * (ptrdiff_t)cs;
@@ -349,6 +350,10 @@ __global__ void __launch_bounds__(128, 4) dslash_fx_kernel(const DslashArgs a, c
         for (int c = 0; c < 3; ++c)
           xch[warp][c][lane] = se > 0 ? make_longlong2(t.lor[c], t.loi[c]) : make_longlong2(-t.lor[c], -t.loi[c]);
         xe[warp][lane][0] = t.E;
+      } else if (QUAD) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) xch[warp][c][lane] = make_longlong2(t.upr[c], t.upi[c]);
+        xe[warp][lane][0] = t.E;
       }
     }
     if ((t.big >> 20) > kFxMaxExp || (t.big != 0 && (t.big >> 20) < kFxMinExp)) t.E = kFxBad;
@@ -357,49 +362,62 @@ __global__ void __launch_bounds__(128, 4) dslash_fx_kernel(const DslashArgs a, c
   __syncthreads();
   double part = 0.0;
   if (act) {
-    Cx<double> acc[6];
-    const unsigned Eo = xe[warp ^ 1][lane][0];
-    // the pair's common unit; kFxBad if either sum is out of range
-    const unsigned E = max(t.E, xe[warp ^ 1][lane][1]);
+    constexpr int NC = QUAD ? 3 : 6;
+    // QUAD: the warp of (x, y) finishes spin sp with the upper sums of (z, t), the
+    // other one spin 2 + sp with the lower ones of spin 1 - sp's (x, y)
+    const int from = !QUAD ? warp ^ 1 : it0 == 0 ? warp ^ 2 : warp ^ 3;
+    const int sp0 = QUAD && it0 ? 2 + sp : sp;
+    Cx<double> acc[NC];
+    // the common unit of the sums; kFxBad if one of the site's is out of range
+    unsigned E = max(t.E, xe[warp ^ 1][lane][1]);
+    if (QUAD) E = max(E, max(xe[warp ^ 2][lane][1], xe[warp ^ 3][lane][1]));
     double unit = __hiloint2double((int)(E - 55u) << 20, 0);  // 2^(E - 1078)
     if (E == kFxBad) {
       Cx<double> all[12];
       hop_sum_f64<DAG>(all, &a.g, a.links, a.c.in, r, par, cb);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        acc[c] = sp == 0 ? all[c] : all[3 + c];
-        acc[3 + c] = sp == 0 ? all[6 + c] : all[9 + c];
+      for (int q = 0; q < NC; ++q) {
+        const int c = q % 3;
+        const Cx<double> u = sp == 0 ? all[c] : all[3 + c], l = sp == 0 ? all[6 + c] : all[9 + c];
+        acc[q] = (QUAD ? it0 != 0 : q >= 3) ? l : u;
       }
       unit = 1.0;
     } else {
-      const unsigned d = E - t.E, dd = E - Eo;
+      const unsigned d = E - t.E, dd = E - xe[from][lane][0];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const longlong2 o = xch[warp ^ 1][c][lane];
-        const long long lr = shr64_s(t.lor[c], d) + shr64_s(o.x, dd), li = shr64_s(t.loi[c], d) + shr64_s(o.y, dd);
-        acc[c] = {(double)shr64_s(t.upr[c], d), (double)shr64_s(t.upi[c], d)};
-        acc[3 + c] = SF > 0 ? Cx<double>{(double)lr, (double)li} : Cx<double>{(double)-lr, (double)-li};
+        const longlong2 o = xch[from][c][lane];
+        if (!QUAD || it0) {
+          const long long lr = shr64_s(t.lor[c], d) + shr64_s(o.x, dd), li = shr64_s(t.loi[c], d) + shr64_s(o.y, dd);
+          acc[NC - 3 + c] = SF > 0 ? Cx<double>{(double)lr, (double)li} : Cx<double>{(double)-lr, (double)-li};
+        } else {
+          acc[c] = {(double)(shr64_s(t.upr[c], d) + shr64_s(o.x, dd)), (double)(shr64_s(t.upi[c], d) + shr64_s(o.y, dd))};
+        }
+        if (!QUAD) acc[c] = {(double)shr64_s(t.upr[c], d), (double)shr64_s(t.upi[c], d)};
       }
     }
     if constexpr (EPI == EPI_OUT) {
       switch (2 * a.c.centre + (a.c.out_inv ? 1 : 0)) {
-        case 0: part = fx_epilogue<EPI, 0, false>(a, sp, r, par, cb, unit, acc); break;
-        case 1: part = fx_epilogue<EPI, 0, true>(a, sp, r, par, cb, unit, acc); break;
-        case 2: part = fx_epilogue<EPI, 1, false>(a, sp, r, par, cb, unit, acc); break;
-        case 3: part = fx_epilogue<EPI, 1, true>(a, sp, r, par, cb, unit, acc); break;
-        case 4: part = fx_epilogue<EPI, 2, false>(a, sp, r, par, cb, unit, acc); break;
-        default: part = fx_epilogue<EPI, 2, true>(a, sp, r, par, cb, unit, acc); break;
+        case 0: part = fx_epilogue<EPI, 0, false>(a, sp0, r, par, cb, unit, acc); break;
+        case 1: part = fx_epilogue<EPI, 0, true>(a, sp0, r, par, cb, unit, acc); break;
+        case 2: part = fx_epilogue<EPI, 1, false>(a, sp0, r, par, cb, unit, acc); break;
+        case 3: part = fx_epilogue<EPI, 1, true>(a, sp0, r, par, cb, unit, acc); break;
+        case 4: part = fx_epilogue<EPI, 2, false>(a, sp0, r, par, cb, unit, acc); break;
+        default: part = fx_epilogue<EPI, 2, true>(a, sp0, r, par, cb, unit, acc); break;
       }
-    } else {  // the solver's operator (launch_one checks the form)
-      part = fx_epilogue<EPI, 2, false>(a, sp, r, par, cb, unit, acc);
+    } else {  // the solver's operator (launch_nr checks the form)
+      part = fx_epilogue<EPI, 2, false>(a, sp0, r, par, cb, unit, acc);
     }
   }
   if (EPI != EPI_OUT || a.c.partial != nullptr) {
     const double ps = warp_sum(part);
     if (lane == 0) xsum[warp] = ps;
     __syncthreads();
-    if (lane == 0 && sp == 0 && r < nrhs && grp < a.nwarp)
-      a.c.partial[((size_t)r * 2 + par) * a.nwarp + grp] = xsum[warp] + xsum[warp + 1];
+    if (lane == 0 && sp == 0 && it0 == 0 && r < nrhs && grp < a.nwarp) {
+      double v = xsum[warp] + xsum[warp + 1];
+      if (QUAD) v += xsum[2] + xsum[3];
+      a.c.partial[((size_t)r * 2 + par) * a.nwarp + grp] = v;
+    }
   }
 }
 

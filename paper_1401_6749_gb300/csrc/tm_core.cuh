@@ -435,6 +435,22 @@ __device__ __forceinline__ Mat3<typename Prec<S>::R> load_link(const void* links
   return U;
 }
 
+// ------------------------------------------------------------- reductions
+// Sum of p[0 .. n - 1] by a block of 256 threads in a fixed order: thread i sums
+// entries i, i + 256, ..., then a fixed tree.  Thread 0 returns the sum.
+__device__ __forceinline__ double block_sum(const double* p, int n) {
+  __shared__ double sh[256];
+  double acc = 0.0;
+  for (int i = threadIdx.x; i < n; i += 256) acc += p[i];
+  sh[threadIdx.x] = acc;
+  __syncthreads();
+  for (int w = 128; w > 0; w >>= 1) {
+    if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+    __syncthreads();
+  }
+  return sh[0];
+}
+
 // ------------------------------------------------------------ bookkeeping
 // While this thread captures a CUDA graph, launches are counted per captured
 // graph (capture_begin / capture_end return how many one replay runs) and are
