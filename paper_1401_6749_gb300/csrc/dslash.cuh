@@ -811,8 +811,8 @@ tm_status_t launch_one(const tm_op* op, const DslashCall& c, cudaStream_t st, in
   a.trace_count = trace_begin(st, &ev);
   if constexpr (HALF && std::is_same<S, double>::value) {
     const int4* lf = static_cast<const int4*>(op->links_fx);
-    if (quad) dslash_fx_kernel<DAG, EPI, true><<<grid, bx, 0, st>>>(a, lf, lgs);
-    else dslash_fx_kernel<DAG, EPI, false><<<grid, bx, 0, st>>>(a, lf, lgs);
+    if (quad) dslash_fx_kernel<EPI, true><<<grid, bx, 0, st>>>(a, lf, lgs);
+    else dslash_fx_kernel<EPI, false><<<grid, bx, 0, st>>>(a, lf, lgs);
   } else if constexpr (HALF) dslash_ff_kernel<DAG, EPI><<<grid, bx, 0, st>>>(a, lgs);
   else if constexpr (MMA) dslash_kernel_mma<S, DAG, EPI><<<grid, kMmaThreads, kMmaSmem, st>>>(a);
   else if constexpr (X2) dslash_kernel_x2<S, RECON, DAG, EPI><<<grid, bx, 0, st>>>(a);

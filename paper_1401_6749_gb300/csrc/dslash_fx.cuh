@@ -171,8 +171,8 @@ __device__ __forceinline__ void fx_hop(FxSum& s, const double2* up, const double
 
 // the hopping sum at site cb of parity par for system r in FP64 arithmetic
 template <bool DAG>
-__device__ __noinline__ void hop_sum_f64(Cx<double>* out, const Geom* gp, const void* links, const void* in, int r,
-                                         int par, int cb) {
+__device__ __forceinline__ void hop_sum_f64_t(Cx<double>* out, const Geom* gp, const void* links, const void* in, int r,
+                                              int par, int cb) {
   const Geom& g = *gp;
   const Site s = site_of(g, par, cb);
   const int opar = par ^ 1;
@@ -196,6 +196,12 @@ __device__ __noinline__ void hop_sum_f64(Cx<double>* out, const Geom* gp, const 
   dir(std::integral_constant<int, 3>{});
 #pragma unroll
   for (int k = 0; k < 12; ++k) out[k] = acc[k];
+}
+
+static __device__ __noinline__ void hop_sum_f64(Cx<double>* out, const Geom* gp, const void* links, const void* in, int r,
+                                         int par, int cb, bool dagger) {
+  if (dagger) hop_sum_f64_t<true>(out, gp, links, in, r, par, cb);
+  else hop_sum_f64_t<false>(out, gp, links, in, r, par, cb);
 }
 
 // The FP64 epilogue (dslash_epilogue) of spin sp0 (acc[0..2]) and, with NC = 6,
@@ -271,14 +277,19 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp0, int 
 // the other one through shared memory.  The loop over (x, y), (z, t) keeps 12
 // sums of 64 bits and the code small.  The pairs of a block take 2^lgs systems
 // (fastest) of the same sites, whose links then come from L1, and the next
-// 32-site groups.  Bound by issue and latency (52% issue-active, 9,100
-// instructions per site and system, of which 1,728 products): 24^3 x 48, 8
-// systems, M: 2.38 ms, FP64 arithmetic 8.15 ms; 4^4, 16 systems 17.3 us against
-// 36.6 us (there one block's chain of instructions).  Measured beside it: one
-// thread per site unrolled over the hops, 2.43 ms and 21.7 us; the input
-// converted once by a pass of its own, 2.19 ms with the pass, 22 us.
-template <bool DAG, int EPI, bool QUAD>
-__global__ void __launch_bounds__(128, 4) dslash_fx_kernel(const DslashArgs a, const int4* links_fx, int lgs) {
+// 32-site groups.
+// Bound by issue and latency (44% issue-active in the solver, 9,100 instructions
+// per site and system, of which 1,728 products): 24^3 x 48, 12 systems, M: 3.48 ms,
+// FP64 arithmetic 12.2 ms.  Measured beside it: three blocks per SM 3.63, four
+// 3.56 or 4.29 ms as the compiler orders the loads (the dagger as a template
+// parameter gave both in one build); one thread per site unrolled over the hops
+// 3.59 ms; the input converted once by a pass of its own 3.25 ms with the pass, but
+// slower on small lattices; four sets of sites per block 3.89 ms (spills).
+// QUAD: four warps take the 32 sites, one for each spin and pair of directions:
+// half the chain of a thread, for lattices that leave SMs idle (4^4, 16 systems:
+// 13.9 us, two warps 17.3, FP64 arithmetic 34.9).
+template <int EPI, bool QUAD>
+__global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const DslashArgs a, const int4* links_fx, int lgs) {
   __shared__ longlong2 xch[4][3][32];
   __shared__ unsigned xe[4][32][2];
   __shared__ double xsum[4];
@@ -286,21 +297,28 @@ __global__ void __launch_bounds__(128, 4) dslash_fx_kernel(const DslashArgs a, c
   const int rg = blockIdx.x % a.rhs_groups;
   const int sb = blockIdx.x / a.rhs_groups;
   const int par = a.c.parity < 0 ? (sb & 1) : a.c.parity;
-  const int gb = a.c.parity < 0 ? (sb >> 1) : sb;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sp = warp & 1, pair = QUAD ? 0 : warp >> 1;
   const int it0 = QUAD ? warp >> 1 : 0, it1 = QUAD ? it0 + 1 : 2;  // pairs of directions of this warp
-  const int grp = QUAD ? gb : gb * (int)(blockDim.x >> (6 + lgs)) + (pair >> lgs);  // 32-site group
+  const int gpb = QUAD ? 1 : (int)(blockDim.x >> (6 + lgs));       // 32-site groups per block
+  const int grp = (a.c.parity < 0 ? (sb >> 1) : sb) * gpb + (pair >> lgs);
   const int cb = grp * 32 + lane;
   const int r = (rg << lgs) + (pair & ((1 << lgs) - 1));
   const int nrhs = a.c.nrhs;
-  const bool act = r < nrhs && (a.c.active == nullptr || a.c.active[r] != 0) && cb < g.Vh;
+  const bool on = r < nrhs && (a.c.active == nullptr || a.c.active[r] != 0);
+  const bool sums = EPI != EPI_OUT || a.c.partial != nullptr;
   if (a.trace_count && blockIdx.x == 0 && threadIdx.x == 0) {
     int n = 0;
     for (int q = 0; q < nrhs; ++q) n += (a.c.active == nullptr || a.c.active[q] != 0) ? 1 : 0;
     *a.trace_count = n;
   }
-  constexpr int SF = DAG ? +1 : -1;
+  const int SF = a.c.dagger ? +1 : -1;  // sign of the forward projection; at run time: one code for M and M^dag
+  if (!__syncthreads_or(on)) {
+    if (sums && lane == 0 && sp == 0 && it0 == 0 && r < nrhs && grp < a.nwarp)
+      a.c.partial[((size_t)r * 2 + par) * a.nwarp + grp] = 0.0;
+    return;
+  }
+  const bool act = on && cb < g.Vh;
   FxSum t;
   if (act) {
     const Site s = site_of(g, par, cb);
@@ -374,7 +392,7 @@ __global__ void __launch_bounds__(128, 4) dslash_fx_kernel(const DslashArgs a, c
     double unit = __hiloint2double((int)(E - 55u) << 20, 0);  // 2^(E - 1078)
     if (E == kFxBad) {
       Cx<double> all[12];
-      hop_sum_f64<DAG>(all, &a.g, a.links, a.c.in, r, par, cb);
+      hop_sum_f64(all, &a.g, a.links, a.c.in, r, par, cb, a.c.dagger);
 #pragma unroll
       for (int q = 0; q < NC; ++q) {
         const int c = q % 3;
@@ -409,8 +427,8 @@ __global__ void __launch_bounds__(128, 4) dslash_fx_kernel(const DslashArgs a, c
       part = fx_epilogue<EPI, 2, false>(a, sp0, r, par, cb, unit, acc);
     }
   }
-  if (EPI != EPI_OUT || a.c.partial != nullptr) {
-    const double ps = warp_sum(part);
+  if (sums) {
+    const double ps = __any_sync(0xffffffffu, act) ? warp_sum(part) : 0.0;
     if (lane == 0) xsum[warp] = ps;
     __syncthreads();
     if (lane == 0 && sp == 0 && it0 == 0 && r < nrhs && grp < a.nwarp) {
