@@ -35,13 +35,12 @@
 
 namespace tml {
 
-tm_status_t xpay(const Geom& g, tm_prec_t prec, void* p, const void* r, const double* beta,
-                 const int* active, int nrhs, int par0, int npar, cudaStream_t s);
+tm_status_t xpay(const Geom& g, tm_prec_t prec, void* p, void* r, const double* beta,
+                 const int* active, int nrhs, int par0, int npar, cudaStream_t s, const XpayRescale& rs);
 tm_status_t fold(const Geom& g, tm_prec_t prec, void* x64, void* y, const double* sigma,
                  const int* mask, int nrhs, int par0, int npar, cudaStream_t s, void* xff = nullptr);
-tm_status_t rescale(const Geom& g, tm_prec_t prec, void* r, const void* r64, const double* sigma,
-                    void* p, const double* ratio, const int* mask, int nrhs, int par0, int npar,
-                    cudaStream_t s, bool r_ff = false);
+tm_status_t rescale(const Geom& g, tm_prec_t prec, void* r, const void* r64, const double* sigma, int nrhs, int par0,
+                    int npar, cudaStream_t s);
 tm_status_t convert_masked(const Geom& g, void* out, tm_prec_t po, const void* in, tm_prec_t pi,
                            int nrhs, const int* active, cudaStream_t s);
 tm_status_t twist(const Geom& g, tm_prec_t prec, void* out, const void* in, double nu, int inverse,
@@ -512,7 +511,7 @@ tm_status_t CgRun::setup() {
   const Half hl = {F / (il ? (size_t)((nrhs + 15) / 16) : (size_t)nrhs), il ? (nrhs + 15) / 16 : nrhs, par0, npar};
   if (mixed) {
     const Half h64 = {F64 / (size_t)nrhs, nrhs, par0, npar};
-    TM_TRY(rescale(g, lo, r, b64, st.sigma, nullptr, nullptr, nullptr, nrhs, par0, npar, s));
+    TM_TRY(rescale(g, lo, r, b64, st.sigma, nrhs, par0, npar, s));
     TM_TRY(half_op(x, nullptr, h64, s));
     TM_TRY(half_op(y, nullptr, hl, s));
     if (ru_ff) {
@@ -550,10 +549,12 @@ tm_status_t CgRun::iteration() {
     e4.out = r64; e4.b = ru_ff ? bff : b64; e4.epi = EPI_RESID; e4.partial = partial; e4.active = st.ru;
     TM_TRY(Op.apply_dag(ru, tmp64, e4));
     TM_TRY(step<CG_RU>());
-    TM_TRY(rescale(g, lo, r, r64, st.sigma, p, st.ratio, st.ru, nrhs, par0, npar, s, ru_ff));
   }
   if (il) return il_xpay(g, lo, xs, p, r, st.alpha, st.beta, st.active, nrhs, par0, npar, s);
-  return xpay(g, lo, p, r, st.beta, st.active, nrhs, par0, npar, s);
+  // p = r + beta p, in mixed solves after rescaling the systems just updated
+  XpayRescale rs;
+  if (mixed) rs = XpayRescale{r64, ru_ff, st.sigma, st.ratio, st.ru};
+  return xpay(g, lo, p, r, st.beta, st.active, nrhs, par0, npar, s, rs);
 }
 
 tm_status_t CgRun::poll() const {

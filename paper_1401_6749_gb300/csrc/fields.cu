@@ -335,22 +335,54 @@ tm_status_t pack_links(const Geom& g, tm_prec_t p, int recon, void* out, const d
 }
 
 // ------------------------------------------------------------ solver BLAS
-// p = r + beta[rhs] p for active systems
-template <class S>
-__global__ void xpay_kernel(Geom g, void* p, const void* r, const double* beta, const int* active,
-                            int nrhs, int par0, int npar) {
+// v 2^k by an integer addition on the exponent, in place of a multiplication on
+// the FP64 pipe: exact in the normal range; denormal results and arguments become
+// zero and results beyond the range infinite (infinities and NaN stay)
+__device__ __forceinline__ double mul_pow2(double v, int k) {
+  const int h = __double2hiint(v), e = (h >> 20) & 0x7ff, n = e + k;
+  const bool zero = e == 0 || (n <= 0 && e != 0x7ff), inf = n >= 0x7ff && e != 0x7ff && e != 0;
+  const int m = h + (e != 0x7ff ? k << 20 : 0);
+  const int sign = h & (int)0x80000000;
+  return __hiloint2double(zero ? sign : inf ? sign | 0x7ff00000 : m, zero || inf ? 0 : __double2loint(v));
+}
+
+// p = r + beta[rhs] p for active systems.  In mixed solves (r64 != null, stored as
+// SR: FP64 or float-float) first the rescaling of the systems whose residual was
+// just recomputed (ru[rhs]): r = r64 / sigma[rhs], p *= ratio[rhs].  sigma and ratio are
+// powers of two, so r is rounded once and p exactly scaled in its own format;
+// one pass, where a launch of its own wrote and read both again (24^3 x 48, 12
+// systems: 141.1 -> 139.5 ms a solve; 16^3 x 32, one system: 6.22 -> 6.04).
+template <class S, class SR>
+__global__ void xpay_kernel(Geom g, void* p, void* r, const double* beta, const int* active, int nrhs, int par0,
+                            int npar, const void* r64, const double* sigma, const double* ratio, const int* ru) {
   const long n = (long)npar * g.Vh;
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n * nrhs) return;
   const int rhs = (int)(i / n);
-  if (!active[rhs]) return;
+  const bool act = active[rhs] != 0, fresh = r64 && ru[rhs] != 0;
+  if (!act && !fresh) return;
   const int rem = (int)(i % n);
-  const size_t b0 = SpinorRef<S>::base(g, rhs, par0 + rem / g.Vh, rem % g.Vh);
+  const int par = par0 + rem / g.Vh, cb = rem % g.Vh;
+  const size_t b0 = SpinorRef<S>::base(g, rhs, par, cb);
   using R = typename Prec<S>::R;
+  if (fresh) {
+    const int k = -ilogb(sigma[rhs]);
+    Cx<double> v[12];
+    load_spinor_f64<SR>(v, r64, SpinorRef<SR>::base(g, rhs, par, cb), (size_t)g.Vh);
+#pragma unroll
+    for (int j = 0; j < 12; ++j) v[j] = {mul_pow2(v[j].re, k), mul_pow2(v[j].im, k)};
+    store_spinor_f64<S>(r, b0, (size_t)g.Vh, v);
+    if (!act) return;
+  }
   const R be = (R)beta[rhs];
   Cx<R> a[12], b[12];
   load_spinor<S>(a, r, b0, (size_t)g.Vh);
   load_spinor<S>(b, p, b0, (size_t)g.Vh);
+  if (fresh) {
+    const R q = (R)ratio[rhs];
+#pragma unroll
+    for (int j = 0; j < 12; ++j) b[j] = q * b[j];
+  }
 #pragma unroll
   for (int j = 0; j < 12; ++j) a[j] = a[j] + be * b[j];
   store_spinor<S>(p, b0, (size_t)g.Vh, a);
@@ -384,59 +416,35 @@ __global__ void fold_kernel(Geom g, void* x64, void* y, const double* sigma, con
   if (xff) store_spinor_f64<FFloat>(xff, SpinorRef<FFloat>::base(g, rhs, par, cb), (size_t)g.Vh, a);
 }
 
-// v 2^k by an integer addition on the exponent, in place of a multiplication on
-// the FP64 pipe: exact in the normal range; denormal results and arguments become
-// zero and results beyond the range infinite (infinities and NaN stay)
-__device__ __forceinline__ double mul_pow2(double v, int k) {
-  const int h = __double2hiint(v), e = (h >> 20) & 0x7ff, n = e + k;
-  const bool zero = e == 0 || (n <= 0 && e != 0x7ff), inf = n >= 0x7ff && e != 0x7ff && e != 0;
-  const int m = h + (e != 0x7ff ? k << 20 : 0);
-  const int sign = h & (int)0x80000000;
-  return __hiloint2double(zero ? sign : inf ? sign | 0x7ff00000 : m, zero || inf ? 0 : __double2loint(v));
-}
-
-// Reliable-update rescaling of the inner iteration (masked systems):
-//   r = r64 / sigma[rhs]   and, if p != null,   p *= ratio[rhs]
-// (r64 stored as SR: FP64, or float-float).  sigma and ratio are powers of two, so
-// r is rounded once and p exactly scaled in its own format.  Bound by memory:
-// with the scales as FP64 factors the FP64 pipe took three times as long
-// (24^3 x 48, 12 systems, FP32: 0.85 ms).
-template <class S, class SR>
-__global__ void rescale_kernel(Geom g, void* r, const void* r64, const double* sigma, void* p,
-                               const double* ratio, const int* mask, int nrhs, int par0, int npar) {
+// r = r64 / sigma[rhs], the inner iteration's first residual (sigma a power of two)
+template <class S>
+__global__ void rescale_kernel(Geom g, void* r, const void* r64, const double* sigma, int nrhs, int par0, int npar) {
   const long n = (long)npar * g.Vh;
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n * nrhs) return;
   const int rhs = (int)(i / n);
-  if (mask && !mask[rhs]) return;
   const int rem = (int)(i % n);
   const int par = par0 + rem / g.Vh, cb = rem % g.Vh;
-  const size_t b64 = SpinorRef<SR>::base(g, rhs, par, cb);
-  const size_t bs = SpinorRef<S>::base(g, rhs, par, cb);
   const int k = -ilogb(sigma[rhs]);
   Cx<double> v[12];
-  load_spinor_f64<SR>(v, r64, b64, (size_t)g.Vh);
+  load_spinor_f64<double>(v, r64, SpinorRef<double>::base(g, rhs, par, cb), (size_t)g.Vh);
 #pragma unroll
   for (int j = 0; j < 12; ++j) v[j] = {mul_pow2(v[j].re, k), mul_pow2(v[j].im, k)};
-  store_spinor_f64<S>(r, bs, (size_t)g.Vh, v);
-  if (p) {
-    using R = typename Prec<S>::R;
-    const R q = (R)ratio[rhs];
-    Cx<R> w[12];
-    load_spinor<S>(w, p, bs, (size_t)g.Vh);
-#pragma unroll
-    for (int j = 0; j < 12; ++j) w[j] = q * w[j];
-    store_spinor<S>(p, bs, (size_t)g.Vh, w);
-  }
+  store_spinor_f64<S>(r, SpinorRef<S>::base(g, rhs, par, cb), (size_t)g.Vh, v);
 }
 
-tm_status_t xpay(const Geom& g, tm_prec_t prec, void* p, const void* r, const double* beta,
-                 const int* active, int nrhs, int par0, int npar, cudaStream_t s) {
+tm_status_t xpay(const Geom& g, tm_prec_t prec, void* p, void* r, const double* beta,
+                 const int* active, int nrhs, int par0, int npar, cudaStream_t s, const XpayRescale& rs) {
   const unsigned nb = blocks_for((long)npar * g.Vh * nrhs, 256);
   TraceScope tr(s, "blas.xpay", 3.0 * 24.0 * prec_size(prec) * npar * g.Vh, 0.0, nrhs);
   return by_prec(prec, [&](auto tag) {
     using S = decltype(tag);
-    xpay_kernel<S><<<nb, 256, 0, s>>>(g, p, r, beta, active, nrhs, par0, npar);
+    if (rs.ff)
+      xpay_kernel<S, FFloat><<<nb, 256, 0, s>>>(g, p, r, beta, active, nrhs, par0, npar, rs.r64, rs.sigma, rs.ratio,
+                                                rs.ru);
+    else
+      xpay_kernel<S, double><<<nb, 256, 0, s>>>(g, p, r, beta, active, nrhs, par0, npar, rs.r64, rs.sigma, rs.ratio,
+                                                rs.ru);
     count_launch();
     return check_launch("xpay");
   });
@@ -453,16 +461,12 @@ tm_status_t fold(const Geom& g, tm_prec_t prec, void* x64, void* y, const double
   });
 }
 
-tm_status_t rescale(const Geom& g, tm_prec_t prec, void* r, const void* r64, const double* sigma,
-                    void* p, const double* ratio, const int* mask, int nrhs, int par0, int npar,
-                    cudaStream_t s, bool r_ff) {
+tm_status_t rescale(const Geom& g, tm_prec_t prec, void* r, const void* r64, const double* sigma, int nrhs, int par0,
+                    int npar, cudaStream_t s) {
   const unsigned nb = blocks_for((long)npar * g.Vh * nrhs, 256);
   return by_prec(prec, [&](auto tag) {
     using S = decltype(tag);
-    if (r_ff)
-      rescale_kernel<S, FFloat><<<nb, 256, 0, s>>>(g, r, r64, sigma, p, ratio, mask, nrhs, par0, npar);
-    else
-      rescale_kernel<S, double><<<nb, 256, 0, s>>>(g, r, r64, sigma, p, ratio, mask, nrhs, par0, npar);
+    rescale_kernel<S><<<nb, 256, 0, s>>>(g, r, r64, sigma, nrhs, par0, npar);
     count_launch();
     return check_launch("rescale");
   });

@@ -128,6 +128,16 @@ struct DslashCall {
   bool il = false;  // fields in the system-interleaved 16-bit layout (dslash_il.cu)
 };
 
+// The rescaling that precedes p = r + beta p in mixed solves (fields.cu); r64 null:
+// none
+struct XpayRescale {
+  const void* r64 = nullptr;
+  bool ff = false;  // r64 in float-float, else FP64
+  const double* sigma = nullptr;
+  const double* ratio = nullptr;
+  const int* ru = nullptr;
+};
+
 inline int nwarp_of(const Geom& g) { return (g.Vh + 31) / 32; }
 
 template <class S, int RECON>
