@@ -75,6 +75,27 @@ __device__ __forceinline__ unsigned fx_row(int cb, int rows) {
   return (unsigned)(cb >> 5) * (unsigned)(32 * rows) + (unsigned)(cb & 31);
 }
 
+// Chunks of a neighbour on their way from memory to the lane's own slots: six
+// 16-byte words (three of spin s, three of 2 + ac), 32 lanes apart
+struct FxStage {
+  double2 w[6][32];
+};
+
+__device__ __forceinline__ void fx_copy(FxStage& st, int lane, const double2* up, const double2* dn, size_t cs) {
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const double2* src = c < 3 ? up + c * cs : dn + (c - 3) * cs;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(&st.w[c][lane])),
+                 "l"(src)
+                 : "memory");
+  }
+}
+__device__ __forceinline__ void fx_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all copies of this thread but those of the last N commits have arrived
+template <int N> __device__ __forceinline__ void fx_arrived() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // The spin structure of a hop, (1 + SGN g_mu) W psi, seen from one upper spin s
 // of the output: h = psi_s + SGN i^ak psi_{2 + ac}, w = W h is added to spin s and
 // SGN i^-ak w to the lower row ac (B_mu A_mu = 1).  In the DeGrand-Rossi basis
@@ -90,16 +111,15 @@ struct FxSum {
 __device__ __forceinline__ long long mad_wide(int a, int b, long long c) { return (long long)a * b + c; }
 
 // one hop: up += w, lo += w (forward) or -= w (backward, W = U^dag), w times -1
-// with nm = -1; up and dn point at the neighbour's chunks of spin s and 2 + ac, u
-// at its link
+// with nm = -1; st holds the neighbour's chunks of spin s and 2 + ac, u points at
+// its link
 template <bool ODD, bool ADJ>
-__device__ __forceinline__ void fx_hop(FxSum& s, const double2* up, const double2* dn, const int4* u, size_t cs,
-                                       int nd, int nm) {
+__device__ __forceinline__ void fx_hop(FxSum& s, const FxStage& st, int lane, const int4* u, int nd, int nm) {
   double2 p[3], q[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    p[c] = up[c * cs];
-    q[c] = dn[c * cs];
+    p[c] = st.w[c][lane];
+    q[c] = st.w[3 + c][lane];
   }
   unsigned big = 0;
 #pragma unroll
@@ -278,18 +298,24 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp0, int 
 // sums of 64 bits and the code small.  The pairs of a block take 2^lgs systems
 // (fastest) of the same sites, whose links then come from L1, and the next
 // 32-site groups.
-// Bound by issue and latency (44% issue-active in the solver, 9,100 instructions
-// per site and system, of which 1,728 products): 24^3 x 48, 12 systems, M: 3.48 ms,
-// FP64 arithmetic 12.2 ms.  Measured beside it: three blocks per SM 3.63, four
-// 3.56 or 4.29 ms as the compiler orders the loads (the dagger as a template
-// parameter gave both in one build); one thread per site unrolled over the hops
-// 3.59 ms; the input converted once by a pass of its own 3.25 ms with the pass, but
-// slower on small lattices; four sets of sites per block 3.89 ms (spills).
+// The neighbours' words come by asynchronous copies to the lane's own slots in
+// shared memory, one hop ahead of the one computed: latency is covered without
+// registers (24^3 x 48, 12 systems, M: loads at their use 3.45 ms, copies 3.29;
+// FP64 arithmetic 12.2.  The same copies for the centre's words 3.40).  No fences
+// or barriers: a lane reads what it copied, and a slot's words are in registers
+// before its next copy starts.
+// Bound by issue and latency (44% issue-active in the solver with the loads at
+// their use; 9,100 instructions per site and system, of which 1,728 products).
+// Measured beside it: four blocks per SM 3.79 ms; one thread per site unrolled
+// over the hops 3.59; four sets of sites per block 3.89 (spills); projections as
+// 64-bit sums 4.8, three products for a complex one 3.38 (the integer pipe is not
+// the bound), products forced to IMAD.WIDE by assembly 4.1.
 // QUAD: four warps take the 32 sites, one for each spin and pair of directions:
 // half the chain of a thread, for lattices that leave SMs idle (4^4, 16 systems:
 // 13.9 us, two warps 17.3, FP64 arithmetic 34.9).
 template <int EPI, bool QUAD>
 __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const DslashArgs a, const int4* links_fx, int lgs) {
+  __shared__ FxStage ring[4][2];
   __shared__ longlong2 xch[4][3][32];
   __shared__ unsigned xe[4][32][2];
   __shared__ double xsum[4];
@@ -325,25 +351,41 @@ __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const Dsla
     const int opar = par ^ 1;
     const size_t cs = (size_t)g.Vh;
     const double2* fup = reinterpret_cast<const double2*>(a.c.in) + ((size_t)(r * 2 + opar) * 12 + 3 * sp) * cs;
+    FxStage &s0 = ring[warp][0], &s1 = ring[warp][1];
+    // the neighbour in direction mu
+    auto nbr = [&](int mu, bool bwd) {
+      const int c = mu & 2 ? (mu & 1 ? s.c[3] : s.c[2]) : (mu & 1 ? s.c[1] : s.c[0]);
+      const int L = g.L[mu], st = g.stride[mu];
+      return (bwd ? (c > 0 ? s.lex - st : s.lex + (L - 1) * st) : (c + 1 < L ? s.lex + st : s.lex - (L - 1) * st)) >> 1;
+    };
+    // start the copy of neighbour n for a hop of pair it
+    auto copy = [&](FxStage& st, int it, int n) {
+      fx_copy(st, lane, fup + n, fup + (6 + 3 * (it ? 0 : 1 - 2 * sp)) * (ptrdiff_t)cs + n, cs);
+    };
     t.E = kFxMinExp;
     t.big = 0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) t.upr[c] = t.upi[c] = 0;
+    copy(s0, it0, nbr(2 * it0, false));
+    fx_commit();
 #pragma unroll 1
     for (int it = it0; it < it1; ++it) {
       const int4* uf = links_fx + (size_t)(4 * it + par) * a.nwarp * 288;  // direction 2 it; the next one: + 576 nwarp
       const int4* ub = links_fx + (size_t)(4 * it + opar) * a.nwarp * 288;
-      const double2* fdn = fup + (6 + 3 * (it ? 0 : 1 - 2 * sp)) * (ptrdiff_t)cs;
       const int so = it && sp ? -1 : 1, se = it || sp ? 1 : -1;  // phase signs: i^ak = so i, se
+      const size_t next = (size_t)a.nwarp * 576;
+      const bool ap = it && g.antiperiodic;
 #pragma unroll
       for (int c = 0; c < 3; ++c) t.lor[c] = t.loi[c] = 0;
-      {
-        const int c = it ? s.c[2] : s.c[0], L = it ? g.L[2] : g.L[0], st = it ? g.stride[2] : 1;
-        const int n1 = (c + 1 < L ? s.lex + st : s.lex - (L - 1) * st) >> 1;
-        const int n2 = (c > 0 ? s.lex - st : s.lex + (L - 1) * st) >> 1;
-        fx_hop<true, false>(t, fup + n1, fdn + n1, uf + fx_row(cb, 9), cs, SF * so >> 1, 0);
-        fx_hop<true, true>(t, fup + n2, fdn + n2, ub + fx_row(n2, 9), cs, -SF * so >> 1, 0);
-      }
+      const int nb0 = nbr(2 * it, true);
+      copy(s1, it, nb0);
+      fx_commit();
+      fx_arrived<1>();
+      fx_hop<true, false>(t, s0, lane, uf + fx_row(cb, 9), SF * so >> 1, 0);
+      copy(s0, it, nbr(2 * it + 1, false));
+      fx_commit();
+      fx_arrived<1>();
+      fx_hop<true, true>(t, s1, lane, ub + fx_row(nb0, 9), -SF * so >> 1, 0);
       // lower row: SF (-so i (w_f - w_b)_odd + se (w_f - w_b)_even); the sums are
       // kept as the bracket times se
 #pragma unroll
@@ -352,17 +394,15 @@ __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const Dsla
         t.lor[c] = so == se ? y : -y;
         t.loi[c] = so == se ? -x : x;
       }
-      {
-        const int c = it ? s.c[3] : s.c[1], L = it ? g.L[3] : g.L[1], st = it ? g.stride[3] : g.stride[1];
-        const int n1 = (c + 1 < L ? s.lex + st : s.lex - (L - 1) * st) >> 1;
-        const int n2 = (c > 0 ? s.lex - st : s.lex + (L - 1) * st) >> 1;
-        const size_t next = (size_t)a.nwarp * 576;
-        const bool ap = it && g.antiperiodic;
-        fx_hop<false, false>(t, fup + n1, fdn + n1, uf + next + fx_row(cb, 9), cs, SF * se >> 1,
-                             ap && c == L - 1 ? -1 : 0);
-        fx_hop<false, true>(t, fup + n2, fdn + n2, ub + next + fx_row(n2, 9), cs, -SF * se >> 1,
-                            ap && c == 0 ? -1 : 0);
-      }
+      const int nb1 = nbr(2 * it + 1, true);
+      copy(s1, it, nb1);
+      fx_commit();
+      fx_arrived<1>();
+      fx_hop<false, false>(t, s0, lane, uf + next + fx_row(cb, 9), SF * se >> 1, ap && s.c[3] == g.L[3] - 1 ? -1 : 0);
+      if (it + 1 < it1) copy(s0, it + 1, nbr(2 * it + 2, false));
+      fx_commit();
+      fx_arrived<1>();
+      fx_hop<false, true>(t, s1, lane, ub + next + fx_row(nb1, 9), -SF * se >> 1, ap && s.c[3] == 0 ? -1 : 0);
       if (it == 0) {  // row 1 - sp
 #pragma unroll
         for (int c = 0; c < 3; ++c)

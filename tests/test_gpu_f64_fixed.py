@@ -38,7 +38,7 @@ def _local_max(psi):
 
 
 @pytest.mark.parametrize("L,n", [((2, 2, 2, 2), 1), ((4, 4, 4, 4), 5), ((6, 4, 2, 10), 3), ((10, 6, 8, 4), 2),
-                                 ((4, 6, 6, 34), 1)])
+                                 ((4, 6, 6, 34), 1), ((4, 6, 6, 34), 3), ((10, 6, 8, 4), 9)])
 @pytest.mark.parametrize("kw", [{}, {"dagger": True}, {"mu_zero": True}])
 def test_ragged(L, n, kw):
     tl = require_gpu()
@@ -50,8 +50,9 @@ def test_ragged(L, n, kw):
     assert np.linalg.norm(got - ref) <= 4e-16 * np.linalg.norm(ref)
 
 
+@pytest.mark.parametrize("n", [2, 14])  # few sites and many: four and two warps per 32 sites
 @pytest.mark.parametrize("decades", [3, 30, 250])
-def test_steep_fields(decades):
+def test_steep_fields(decades, n):
     """Neighbouring sites of very unlike size: the error follows the largest
     component of each stencil (beyond 2^-863 .. 2^878 the FP64 arithmetic)."""
     tl = require_gpu()
@@ -59,22 +60,23 @@ def test_steep_fields(decades):
     U = synth.gauge_field(L, 6)
     op = tl.Operator(L, KAPPA, MU, to_dev(U))
     rng = np.random.default_rng(3)
-    scale = 10.0 ** rng.uniform(-decades, decades, size=(2,) + site_shape(L))
+    scale = 10.0 ** rng.uniform(-decades, decades, size=(n,) + site_shape(L))
     scale[:, 1, :2] = 0.0  # zero sites among them
-    psi = synth.random_spinor(L, 2, 11) * scale[..., None, None]
+    psi = synth.random_spinor(L, n, 11) * scale[..., None, None]
     got = _apply(tl, op, L, psi)
     ref = oop.apply_M(U, psi, KAPPA, MU)
     err = np.abs(got - ref).max(axis=(-1, -2))
     assert np.all(err <= 1.5e-14 * _local_max(psi))
 
 
-def test_special_values():
+@pytest.mark.parametrize("n", [3, 24])
+def test_special_values(n):
     """Infinities and NaN reach the sites that read them and no others."""
     tl = require_gpu()
     L = (4, 4, 4, 8)
     U = synth.gauge_field(L, 7)
     op = tl.Operator(L, KAPPA, MU, to_dev(U))
-    psi = synth.random_spinor(L, 3, 12)
+    psi = synth.random_spinor(L, n, 12)
     clean = _apply(tl, op, L, psi)
     bad = psi.copy()
     bad[1, 2, 1, 0, 3, 1, 2] = np.inf

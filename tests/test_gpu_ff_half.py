@@ -18,7 +18,8 @@ pytestmark = pytest.mark.gpu
 KAPPA, MU = 0.16, 0.02
 
 
-@pytest.mark.parametrize("L,n", [((2, 2, 2, 2), 1), ((6, 4, 2, 10), 3), ((4, 6, 6, 34), 1), ((10, 6, 8, 4), 2)])
+@pytest.mark.parametrize("L,n", [((2, 2, 2, 2), 1), ((6, 4, 2, 10), 3), ((4, 6, 6, 34), 1), ((10, 6, 8, 4), 2),
+                                 ((10, 6, 8, 4), 9)])
 @pytest.mark.parametrize("kw", [{}, {"dagger": True}, {"mu_zero": True}])
 @pytest.mark.parametrize("anti", [True, False])
 def test_forms(L, n, kw, anti):
