@@ -304,8 +304,8 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp0, int 
 // FP64 arithmetic 12.2.  The same copies for the centre's words 3.40).  No fences
 // or barriers: a lane reads what it copied, and a slot's words are in registers
 // before its next copy starts.
-// Bound by issue and latency (44% issue-active in the solver with the loads at
-// their use; 9,100 instructions per site and system, of which 1,728 products).
+// Bound by the integer multiplier (67% busy), fixed latencies of the 64-bit sums and
+// issue (53% active): 9,100 instructions per site and system, of which 1,728 products.
 // Measured beside it: four blocks per SM 3.79 ms; one thread per site unrolled
 // over the hops 3.59; four sets of sites per block 3.89 (spills); projections as
 // 64-bit sums 4.8, three products for a complex one 3.38 (the integer pipe is not
