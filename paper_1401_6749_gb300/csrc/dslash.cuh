@@ -774,7 +774,7 @@ tm_status_t launch_one(const tm_op* op, const DslashCall& c, cudaStream_t st, in
   bool quad = false;
   if constexpr (HALF) {
     // pairs of warps, two to a block; where there are too few for every SM,
-    // four warps per 32 sites (FP64) or one pair to a block
+    // four warps per 32 sites (FP64, the same bits) or one pair to a block
     const long pairs = (long)a.nwarp * (c.parity < 0 ? 2 : 1) * c.nrhs;
     const bool few = pairs < 2 * 152;
     quad = few && std::is_same<S, double>::value;

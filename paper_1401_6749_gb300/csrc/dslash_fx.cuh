@@ -27,6 +27,11 @@
 // site to an FP64 evaluation of the same sum (hop_sum_f64), so the kernel's
 // range and special values are those of the FP64 arithmetic.
 //
+// The hops of (x, y) and those of (z, t) are summed apart, each pair of
+// directions in a unit of its own, and brought to the larger unit at the end:
+// so two and four warps per 32 sites (dslash_fx_kernel) compute the same bits, and
+// a system's result does not depend on how many share the launch.
+//
 // The sums T are converted to FP64 once per output component; centre, twist
 // and CG update follow in FP64 (fx_epilogue).
 #pragma once
@@ -251,7 +256,7 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp0, int 
       o[q] = {shop * v.re, shop * v.im};
     }
   }
-  double part = 0.0;
+  double part[2] = {0.0, 0.0};  // of the two spins
   if constexpr (EPI == EPI_OUT) {
     double2* out = reinterpret_cast<double2*>(a.c.out) + b0;
 #pragma unroll
@@ -261,7 +266,7 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp0, int 
     }
     if (a.c.partial) {
 #pragma unroll
-      for (int q = 0; q < NC; ++q) part = __fma_rn(o[q].re, o[q].re, __fma_rn(o[q].im, o[q].im, part));
+      for (int q = 0; q < NC; ++q) part[q / 3] = __fma_rn(o[q].re, o[q].re, __fma_rn(o[q].im, o[q].im, part[q / 3]));
     }
   } else if constexpr (EPI == EPI_CGUPD) {
     const double al = a.c.alpha[r];
@@ -275,7 +280,7 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp0, int 
       const double2 n = make_double2(__fma_rn(-al, o[q].re, v.x), __fma_rn(-al, o[q].im, v.y));
       rf[i] = n;
       xf[i] = make_double2(__fma_rn(al, p.x, x.x), __fma_rn(al, p.y, x.y));
-      part = __fma_rn(n.x, n.x, __fma_rn(n.y, n.y, part));
+      part[q / 3] = __fma_rn(n.x, n.x, __fma_rn(n.y, n.y, part[q / 3]));
     }
   } else {  // EPI_RESID
     const double2* bf = reinterpret_cast<const double2*>(a.c.b) + b0;
@@ -286,16 +291,17 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp0, int 
       const double2 v = bf[i];
       const double2 n = make_double2(__dsub_rn(v.x, o[q].re), __dsub_rn(v.y, o[q].im));
       out[i] = n;
-      part = __fma_rn(n.x, n.x, __fma_rn(n.y, n.y, part));
+      part[q / 3] = __fma_rn(n.x, n.x, __fma_rn(n.y, n.y, part[q / 3]));
     }
   }
-  return part;
+  return NC == 6 ? __dadd_rn(part[0], part[1]) : part[0];
 }
 
 // Two warps take 32 consecutive sites of one system, one for each upper spin
 // (with the lower rows it feeds), and exchange the lower row that belongs to
 // the other one through shared memory.  The loop over (x, y), (z, t) keeps 12
-// sums of 64 bits and the code small.  The pairs of a block take 2^lgs systems
+// sums of 64 bits and the code small; the upper sums of (x, y) wait in shared
+// memory too.  The pairs of a block take 2^lgs systems
 // (fastest) of the same sites, whose links then come from L1, and the next
 // 32-site groups.
 // The neighbours' words come by asynchronous copies to the lane's own slots in
@@ -316,9 +322,10 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp0, int 
 template <int EPI, bool QUAD>
 __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const DslashArgs a, const int4* links_fx, int lgs) {
   __shared__ FxStage ring[4][2];
-  __shared__ longlong2 xch[4][3][32];
-  __shared__ unsigned xe[4][32][2];
+  __shared__ longlong2 xu[4][3][32], xl[4][3][32];  // upper and lower sums on their way to another warp or loop
+  __shared__ unsigned xe[2][4][32];                 // units of [pair of warps][2 upper spin + pair of directions]
   __shared__ double xsum[4];
+  __shared__ double xpart[2][32];
   const Geom& g = a.g;
   const int rg = blockIdx.x % a.rhs_groups;
   const int sb = blockIdx.x / a.rhs_groups;
@@ -362,10 +369,6 @@ __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const Dsla
     auto copy = [&](FxStage& st, int it, int n) {
       fx_copy(st, lane, fup + n, fup + (6 + 3 * (it ? 0 : 1 - 2 * sp)) * (ptrdiff_t)cs + n, cs);
     };
-    t.E = kFxMinExp;
-    t.big = 0;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) t.upr[c] = t.upi[c] = 0;
     copy(s0, it0, nbr(2 * it0, false));
     fx_commit();
 #pragma unroll 1
@@ -376,7 +379,9 @@ __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const Dsla
       const size_t next = (size_t)a.nwarp * 576;
       const bool ap = it && g.antiperiodic;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) t.lor[c] = t.loi[c] = 0;
+      for (int c = 0; c < 3; ++c) t.upr[c] = t.upi[c] = t.lor[c] = t.loi[c] = 0;
+      t.E = kFxMinExp;
+      t.big = 0;
       const int nb0 = nbr(2 * it, true);
       copy(s1, it, nb0);
       fx_commit();
@@ -406,16 +411,15 @@ __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const Dsla
       if (it == 0) {  // row 1 - sp
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-          xch[warp][c][lane] = se > 0 ? make_longlong2(t.lor[c], t.loi[c]) : make_longlong2(-t.lor[c], -t.loi[c]);
-        xe[warp][lane][0] = t.E;
-      } else if (QUAD) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) xch[warp][c][lane] = make_longlong2(t.upr[c], t.upi[c]);
-        xe[warp][lane][0] = t.E;
+          xl[warp][c][lane] = se > 0 ? make_longlong2(t.lor[c], t.loi[c]) : make_longlong2(-t.lor[c], -t.loi[c]);
       }
+      if (QUAD ? it != 0 : it == 0) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) xu[warp][c][lane] = make_longlong2(t.upr[c], t.upi[c]);
+      }
+      if ((t.big >> 20) > kFxMaxExp || (t.big != 0 && (t.big >> 20) < kFxMinExp)) t.E = kFxBad;
+      xe[pair][2 * sp + it][lane] = t.E;
     }
-    if ((t.big >> 20) > kFxMaxExp || (t.big != 0 && (t.big >> 20) < kFxMinExp)) t.E = kFxBad;
-    xe[warp][lane][1] = t.E;
   }
   __syncthreads();
   double part = 0.0;
@@ -423,12 +427,13 @@ __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const Dsla
     constexpr int NC = QUAD ? 3 : 6;
     // QUAD: the warp of (x, y) finishes spin sp with the upper sums of (z, t), the
     // other one spin 2 + sp with the lower ones of spin 1 - sp's (x, y)
-    const int from = !QUAD ? warp ^ 1 : it0 == 0 ? warp ^ 2 : warp ^ 3;
     const int sp0 = QUAD && it0 ? 2 + sp : sp;
     Cx<double> acc[NC];
-    // the common unit of the sums; kFxBad if one of the site's is out of range
-    unsigned E = max(t.E, xe[warp ^ 1][lane][1]);
-    if (QUAD) E = max(E, max(xe[warp ^ 2][lane][1], xe[warp ^ 3][lane][1]));
+    // the common unit of the site's sums; kFxBad if one of them is out of range
+    unsigned e[2][2];  // [this or the other upper spin][pair of directions]
+#pragma unroll
+    for (int j = 0; j < 4; ++j) e[j >> 1][j & 1] = xe[pair][2 * (sp ^ (j >> 1)) + (j & 1)][lane];
+    const unsigned E = max(max(e[0][0], e[0][1]), max(e[1][0], e[1][1]));
     double unit = __hiloint2double((int)(E - 55u) << 20, 0);  // 2^(E - 1078)
     if (E == kFxBad) {
       Cx<double> all[12];
@@ -441,17 +446,19 @@ __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const Dsla
       }
       unit = 1.0;
     } else {
-      const unsigned d = E - t.E, dd = E - xe[from][lane][0];
+      const unsigned d0 = E - e[0][0], d1 = E - e[0][1], dx = E - e[1][0];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const longlong2 o = xch[from][c][lane];
-        if (!QUAD || it0) {
-          const long long lr = shr64_s(t.lor[c], d) + shr64_s(o.x, dd), li = shr64_s(t.loi[c], d) + shr64_s(o.y, dd);
-          acc[NC - 3 + c] = SF > 0 ? Cx<double>{(double)lr, (double)li} : Cx<double>{(double)-lr, (double)-li};
-        } else {
-          acc[c] = {(double)(shr64_s(t.upr[c], d) + shr64_s(o.x, dd)), (double)(shr64_s(t.upi[c], d) + shr64_s(o.y, dd))};
+        if (!QUAD || it0 == 0) {
+          const longlong2 o = xu[QUAD ? warp ^ 2 : warp][c][lane];  // QUAD: of (z, t), else of (x, y)
+          const unsigned dt = QUAD ? d0 : d1, dd = QUAD ? d1 : d0;
+          acc[c] = {(double)(shr64_s(t.upr[c], dt) + shr64_s(o.x, dd)), (double)(shr64_s(t.upi[c], dt) + shr64_s(o.y, dd))};
         }
-        if (!QUAD) acc[c] = {(double)shr64_s(t.upr[c], d), (double)shr64_s(t.upi[c], d)};
+        if (!QUAD || it0) {
+          const longlong2 o = xl[QUAD ? warp ^ 3 : warp ^ 1][c][lane];
+          const long long lr = shr64_s(t.lor[c], d1) + shr64_s(o.x, dx), li = shr64_s(t.loi[c], d1) + shr64_s(o.y, dx);
+          acc[NC - 3 + c] = SF > 0 ? Cx<double>{(double)lr, (double)li} : Cx<double>{(double)-lr, (double)-li};
+        }
       }
     }
     if constexpr (EPI == EPI_OUT) {
@@ -468,14 +475,18 @@ __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const Dsla
     }
   }
   if (sums) {
+    // per site first the upper and the lower spin's terms, then the warp's sites,
+    // then the spins: in this order in both forms
+    if constexpr (QUAD) {
+      if (it0) xpart[sp][lane] = part;
+      __syncthreads();
+      if (it0 == 0) part += xpart[sp][lane];
+    }
     const double ps = __any_sync(0xffffffffu, act) ? warp_sum(part) : 0.0;
     if (lane == 0) xsum[warp] = ps;
     __syncthreads();
-    if (lane == 0 && sp == 0 && it0 == 0 && r < nrhs && grp < a.nwarp) {
-      double v = xsum[warp] + xsum[warp + 1];
-      if (QUAD) v += xsum[2] + xsum[3];
-      a.c.partial[((size_t)r * 2 + par) * a.nwarp + grp] = v;
-    }
+    if (lane == 0 && sp == 0 && it0 == 0 && r < nrhs && grp < a.nwarp)
+      a.c.partial[((size_t)r * 2 + par) * a.nwarp + grp] = xsum[warp] + xsum[warp + 1];
   }
 }
 

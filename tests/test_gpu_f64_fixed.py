@@ -98,3 +98,39 @@ def test_links_out_of_range():
     psi = synth.random_spinor(L, 2, 13)
     ref = oop.apply_M(U, psi, KAPPA, MU)
     assert np.linalg.norm(_apply(tl, op, L, psi) - ref) <= 1e-15 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("kw", [{}, {"dagger": True}, {"mu_zero": True}])
+def test_batch_independence(kw):
+    """A system alone (four warps per 32 sites) and among enough others for two:
+    the same bits."""
+    tl = require_gpu()
+    L, n = (8, 8, 8, 16), 5
+    op = tl.Operator(L, KAPPA, MU, to_dev(synth.gauge_field(L, 21)))
+    psi = synth.random_spinor(L, n, 22)
+    psi[3] *= 10.0 ** np.random.default_rng(1).uniform(-3, 3, size=site_shape(L))[..., None, None]
+    many = _apply(tl, op, L, psi, **kw)
+    for j in (0, 3):
+        np.testing.assert_array_equal(_apply(tl, op, L, psi[j:j + 1], **kw)[0], many[j])
+
+
+@pytest.mark.parametrize("mode", ["plain", "mixed"])
+def test_solve_batch_independence(mode):
+    """The CG updates, residuals and norms too."""
+    tl = require_gpu()
+    L, n = (8, 8, 8, 16), 5
+    op = tl.Operator(L, KAPPA, MU, to_dev(synth.gauge_field(L, 21)))
+    m = tl.CG_PLAIN if mode == "plain" else tl.CG_MIXED
+    par = tl.cg_params(1e-10, 500, m, prec=tl.F64, inner_prec=tl.F32, schur=True, true_residual=True)
+
+    def solve(first, k):
+        eta, x = tl.empty_field(L, tl.F64, k), tl.empty_field(L, tl.F64, k)
+        tl.z4_noise(L, eta, tl.F64, 7, first, k)
+        _, stats = tl.tm_cg_solve(op, x, eta, k, par)
+        return unpack(tl, L, x, tl.F64, k), stats
+
+    many, stats = solve(0, n)
+    for j in (0, 4):
+        one, s1 = solve(j, 1)
+        np.testing.assert_array_equal(one[0], many[j])
+        assert s1[0] == stats[j]
