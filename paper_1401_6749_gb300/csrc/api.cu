@@ -301,7 +301,8 @@ size_t link_bytes(const Geom& g, tm_prec_t p, int recon);
 tm_status_t pack_links(const Geom& g, tm_prec_t p, int recon, void* out, const double* U,
                        cudaStream_t s);
 size_t links_fx_bytes(const Geom& g);
-tm_status_t pack_links_fx(const Geom& g, void* out, const double* U, int* bad, cudaStream_t s);
+tm_status_t pack_links_fx(const Geom& g, void* out, const double* U, unsigned long long* stat, cudaStream_t s);
+bool links_fx_ok(const unsigned long long* stat);
 
 }  // namespace tml
 
@@ -524,17 +525,17 @@ extern "C" tm_status_t tm_op_create(tm_op_t** out, const tm_params_t* p, const d
       }
     }
   }
-  // fixed-point copy for the FP64 Dslash; *fx_bad tells whether every link is in its range
-  int* fx_bad = nullptr;
-  int h_bad = 0;
+  // fixed-point copy for the FP64 Dslash, and whether it takes these links
+  unsigned long long* fx_stat = nullptr;
+  unsigned long long h_stat[3] = {0, 0, 0};
   {
     tm_status_t s5 = dev_alloc(&op->links_fx, links_fx_bytes(op->g), st, "tm_op_create");
-    if (s5 == TM_OK) s5 = dev_alloc((void**)&fx_bad, sizeof(int), st, "tm_op_create");
-    if (s5 == TM_OK && cudaMemsetAsync(fx_bad, 0, sizeof(int), st) != cudaSuccess) s5 = TM_ERR_CUDA;
-    if (s5 == TM_OK) s5 = pack_links_fx(op->g, op->links_fx, U, fx_bad, st);
-    if (s5 == TM_OK && cudaMemcpyAsync(&h_bad, fx_bad, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+    if (s5 == TM_OK) s5 = dev_alloc((void**)&fx_stat, sizeof(h_stat), st, "tm_op_create");
+    if (s5 == TM_OK && cudaMemsetAsync(fx_stat, 0, sizeof(h_stat), st) != cudaSuccess) s5 = TM_ERR_CUDA;
+    if (s5 == TM_OK) s5 = pack_links_fx(op->g, op->links_fx, U, fx_stat, st);
+    if (s5 == TM_OK && cudaMemcpyAsync(h_stat, fx_stat, sizeof(h_stat), cudaMemcpyDeviceToHost, st) != cudaSuccess)
       s5 = TM_ERR_CUDA;
-    dev_free(fx_bad, st);
+    dev_free(fx_stat, st);
     if (s5 != TM_OK) {
       if (s5 == TM_ERR_CUDA) cudaGetLastError();
       dev_free(staged, st);
@@ -553,7 +554,7 @@ extern "C" tm_status_t tm_op_create(tm_op_t** out, const tm_params_t* p, const d
     tm_op_destroy(op);
     return TM_ERR_CUDA;
   }
-  if (h_bad) {
+  if (!links_fx_ok(h_stat)) {
     dev_free(op->links_fx, st);
     op->links_fx = nullptr;
   }

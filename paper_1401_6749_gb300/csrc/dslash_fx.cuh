@@ -6,31 +6,43 @@
 // reals are added with factors of modulus <= 1, so a fixed point relative to
 // the largest of them keeps more bits than FP64 rounding of the partial sums.
 //
-// With E one above the biased exponent of the largest component met so far, a
-// component x enters as F = trunc(x 2^(1078 - E)), |F| < 2^56, split into hi 2^27 +
-// lo (both with the sign of x).  A link's part u is round(u 2^54) = ghi 2^27 + glo,
-// |glo| <= 2^26 (pack_links_fx, made with the operator; |u| <= 1.25 is checked
-// there, other links take the FP64 kernel).  Spin projections are integer
-// sums of the halves and every product F G is three IMAD.WIDE:
+// With E at least the biased exponent of the largest component met so far (one
+// above it where it was raised), a component x enters as F = trunc(x 2^(1080 - E)),
+// |F| < 2^58, split into hi 2^29 + lo (both with the sign of x).  A link's part u is
+// round(u 2^58) = ghi 2^29 + glo, |glo| <= 2^28 (pack_links_fx, made with the
+// operator, which also says which links the fixed point takes).  Spin projections
+// are integer sums of the halves and every product F G is three IMAD.WIDE:
 //   hh += ghi hi,   md += ghi lo + glo hi        (glo lo, below the unit, is dropped)
-// A hop adds T = hh + (md >> 27) in units of 2^(E - 1078), 2^-56 of the bound
-// 2^(E - 1022) on the components.  |hi| < 2^30 and |lo| < 2^28 after the
-// projection, so the sum over 8 hops, 3 colours and 2 parts stays below
-// 48 * 1.25 * 2^57 < 2^63.  Rounding: inputs truncated at 2^-56 of the bound, links
-// 2^-55 of the factor, a unit of dropped products per term at most: a few
-// 2^-55 of the largest component of the stencil, below what the 60 roundings of
-// an FP64 evaluation leave (2^-53 of a partial sum each).  Measured against
-// complex128: M 1.14e-16 (FP64 arithmetic 1.36e-16), four hopping-expansion
-// steps 2.96e-16 (3.08e-16).
-//
-// Components outside 2^-863 .. 2^878 (infinities and NaN among them) send the
-// site to an FP64 evaluation of the same sum (hop_sum_f64), so the kernel's
-// range and special values are those of the FP64 arithmetic.
+// A hop adds T = hh + (md >> 29) in units of 2^(E - 1080), 2^-58 of the bound
+// B = 2^(E - 1022) on the components.  |hi| < 2^30 and |lo| < 2^30 after the
+// projection.  Rows of a link have norms of at most 1.5, so by Cauchy and Schwarz the
+// sums over a row stay below 1.5 sqrt(6) 2^59 (hh, T) and 2^62 (md), and those over
+// four hops below 2^63.
 //
 // The hops of (x, y) and those of (z, t) are summed apart, each pair of
-// directions in a unit of its own, and brought to the larger unit at the end:
+// directions in a unit of its own, and brought to twice the larger unit at the end:
 // so two and four warps per 32 sites (dslash_fx_kernel) compute the same bits, and
 // a system's result does not depend on how many share the launch.
+//
+// Error, in units: per hop 2.5 |row| from the inputs (only those below B / 32 lose
+// bits), 6 from the dropped products, 1.5 |row| from the links, 1 from the rounding of T
+// and the shifts: at most 125 in all, 3.9 B 2^-53, where FP64 arithmetic errs by up
+// to some 50 roundings of the terms that it adds.  These may be far below B: one
+// colour small against another with links that hardly mix them, or one neighbour far
+// larger than the others.  FP64 keeps the digits of such a component and this sum
+// would not, so S, the sum of |re w| + |im w| over the hops, w = W h, is added up beside
+// it (FxSum::s) and a site where that is less than B / 4 for any spin and colour takes
+// FP64 sums instead (fx_sums_f64).  Replayed in integers against extended precision
+// (links exp(i eps H), eps = 0 .. 2; Gaussian fields, steep ones, colours of unlike
+// size), the rms error is 0.35 to 0.5 of that of FP64 arithmetic in all, and in the
+// components with S between B / 4 and B / 2, the worst, 0.5 to 1.2 of it (B / 8 to B / 4: 0.8 to 2).
+// Gaussian fields, CG vectors, Z4 sources and solutions of them have S > B / 4 at every
+// site.  M at 16^3 x 32 against complex128: 1.1e-16 (FP64 arithmetic 1.36e-16), of which
+// the centre and the last rounding are the most.
+//
+// Components outside 2^-863 .. 2^878 (infinities and NaN among them) send the
+// site to the same FP64 sums, so the kernel's range and special values are those of
+// the FP64 arithmetic.
 //
 // The sums T are converted to FP64 once per output component; centre, twist
 // and CG update follow in FP64 (fx_epilogue).
@@ -40,9 +52,14 @@
 namespace tml {
 
 constexpr unsigned kFxMinExp = 160, kFxMaxExp = 1900;  // biased exponents the fixed point takes
-constexpr unsigned kFxBad = 0x7fffu;                   // mark of a sum out of that range
+constexpr unsigned kFxBad = 0x7fffu;                   // mark of a site that takes FP64 sums
 
-// right shifts, zero / the sign for counts of 64 and more
+// right shifts, zero / the sign for counts of the width and more
+__device__ __forceinline__ unsigned shr32(unsigned v, unsigned n) {
+  unsigned r;
+  asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
+  return r;
+}
 __device__ __forceinline__ unsigned shr64_lo(unsigned long long v, unsigned n) {
   unsigned long long r;
   asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
@@ -54,14 +71,14 @@ __device__ __forceinline__ long long shr64_s(long long v, unsigned n) {
   return r;
 }
 
-// |x| 2^(1078 - E) truncated, as unsigned halves (hi, lo < 2^27); z: +-1, x's sign
+// |x| 2^(1080 - E) truncated, as unsigned halves (hi, lo < 2^29); z: +-1, x's sign
 // times that of the mask nm (0 or -1)
 __device__ __forceinline__ int3 fx_of(double x, unsigned E, int nm) {
   const int h = __double2hiint(x);
   const unsigned long long m =
-      ((unsigned long long)(((unsigned)h & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(x)) << 3;
+      ((unsigned long long)(((unsigned)h & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(x)) << 5;
   const unsigned sh = E - (((unsigned)h >> 20) & 0x7ffu);
-  return make_int3((int)shr64_lo(m, sh + 27), (int)(shr64_lo(m, sh) & 0x7ffffffu), ((h >> 31) ^ nm) | 1);
+  return make_int3((int)shr64_lo(m, sh + 29), (int)(shr64_lo(m, sh) & 0x1fffffffu), ((h >> 31) ^ nm) | 1);
 }
 
 struct Fx {
@@ -109,8 +126,9 @@ template <int N> __device__ __forceinline__ void fx_arrived() {
 // mask nd (0 or -1) on psi_{2 + ac}.
 struct FxSum {
   long long upr[3], upi[3], lor[3], loi[3];
-  unsigned E;    // units of 2^(E - 1078)
-  unsigned big;  // largest |high word| met
+  unsigned s[3];  // sum of |re w| + |im w| over the hops, in units of 2^-26 B
+  unsigned E;     // units of 2^(E - 1080)
+  unsigned big;   // largest |high word| met
 };
 
 __device__ __forceinline__ long long mad_wide(int a, int b, long long c) { return (long long)a * b + c; }
@@ -147,6 +165,7 @@ __device__ __forceinline__ void fx_hop(FxSum& s, const FxStage& st, int lane, co
       s.upi[a] = shr64_s(s.upi[a], d);
       s.lor[a] = shr64_s(s.lor[a], d);
       s.loi[a] = shr64_s(s.loi[a], d);
+      s.s[a] = shr32(s.s[a], d);
     }
     s.E = E;
   }
@@ -165,9 +184,8 @@ __device__ __forceinline__ void fx_hop(FxSum& s, const FxStage& st, int lane, co
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     // re: u.re h.re - u.im h.im,  im: u.re h.im + u.im h.re  (u.im -> -u.im for the adjoint)
-    // md starts at half a unit, so that md >> 27 rounds (rounding down doubles
-    // the error of a solve, 1.2e-15 against 5.7e-16 at 4^4)
-    long long hr = 0, hi = 0, mr = 1 << 26, mi = 1 << 26;
+    // md starts at half a unit, so that md >> 29 rounds
+    long long hr = 0, hi = 0, mr = 1 << 28, mi = 1 << 28;
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
       const int4 w = u[(ADJ ? 3 * b + a : 3 * a + b) * 32];  // (re.hi, re.lo, im.hi, im.lo)
@@ -186,7 +204,8 @@ __device__ __forceinline__ void fx_hop(FxSum& s, const FxStage& st, int lane, co
       mr = mad_wide(w.w, si.hi, mr);
       mi = mad_wide(w.w, sr.hi, mi);
     }
-    const long long tr = hr + (mr >> 27), ti = hi + (mi >> 27);
+    const long long tr = hr + (mr >> 29), ti = hi + (mi >> 29);
+    s.s[a] += (unsigned)abs((int)(tr >> 32)) + (unsigned)abs((int)(ti >> 32));
     s.upr[a] += tr;
     s.upi[a] += ti;
     s.lor[a] += ADJ ? -tr : tr;
@@ -194,39 +213,102 @@ __device__ __forceinline__ void fx_hop(FxSum& s, const FxStage& st, int lane, co
   }
 }
 
-// the hopping sum at site cb of parity par for system r in FP64 arithmetic
-template <bool DAG>
-__device__ __forceinline__ void hop_sum_f64_t(Cx<double>* out, const Geom* gp, const void* links, const void* in, int r,
-                                              int par, int cb) {
-  const Geom& g = *gp;
-  const Site s = site_of(g, par, cb);
-  const int opar = par ^ 1;
-  const size_t cs = (size_t)g.Vh, f0 = (size_t)(r * 2 + opar) * 12 * cs;
-  Cx<double> acc[12];
+// One hop in FP64 arithmetic, as fx_hop: up += w, lo +- w; sd and sw (+-1) multiply
+// psi_{2 + ac} and w
+template <bool ODD, bool ADJ>
+__device__ __forceinline__ void f64_hop(Cx<double> (&up)[3], Cx<double> (&lo)[3], const double2* pu, const double2* pd,
+                                        const double2* u, size_t cs, double sd, double sw) {
+  Cx<double> h[3];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = {0.0, 0.0};
-  constexpr int SF = DAG ? +1 : -1, SB = -SF;
-  auto dir = [&](auto mu_tag) {
-    constexpr int MU = decltype(mu_tag)::value;
-    const bool edge = MU == 3 && g.antiperiodic;
-    const int lf = lex_fwd(g, s, MU) >> 1, lb = lex_bwd(g, s, MU) >> 1;
-    hop_site<double, MU, SF, false>(acc, in, f0 + lf, cs, load_link<double, 18>(links, g, MU, par, cb),
-                                    edge && s.c[3] == g.L[3] - 1 ? -1.0 : 1.0);
-    hop_site<double, MU, SB, true>(acc, in, f0 + lb, cs, load_link<double, 18>(links, g, MU, opar, lb),
-                                   edge && s.c[3] == 0 ? -1.0 : 1.0);
-  };
-  dir(std::integral_constant<int, 0>{});
-  dir(std::integral_constant<int, 1>{});
-  dir(std::integral_constant<int, 2>{});
-  dir(std::integral_constant<int, 3>{});
+  for (int c = 0; c < 3; ++c) {
+    const double2 p = pu[c * cs], q = pd[c * cs];
+    if constexpr (ODD) h[c] = {sw * __fma_rn(-sd, q.y, p.x), sw * __fma_rn(sd, q.x, p.y)};
+    else h[c] = {sw * __fma_rn(sd, q.x, p.x), sw * __fma_rn(sd, q.y, p.y)};
+  }
 #pragma unroll
-  for (int k = 0; k < 12; ++k) out[k] = acc[k];
+  for (int a = 0; a < 3; ++a) {
+    double zr = 0.0, zi = 0.0;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const double2 v = u[(ADJ ? 3 * b + a : 3 * a + b) * cs];
+      const double vi = ADJ ? -v.y : v.y;
+      zr = __fma_rn(v.x, h[b].re, zr);
+      zr = __fma_rn(-vi, h[b].im, zr);
+      zi = __fma_rn(v.x, h[b].im, zi);
+      zi = __fma_rn(vi, h[b].re, zi);
+    }
+    up[a] = {__dadd_rn(up[a].re, zr), __dadd_rn(up[a].im, zi)};
+    lo[a] = ADJ ? Cx<double>{__dsub_rn(lo[a].re, zr), __dsub_rn(lo[a].im, zi)}
+                : Cx<double>{__dadd_rn(lo[a].re, zr), __dadd_rn(lo[a].im, zi)};
+  }
 }
 
-static __device__ __noinline__ void hop_sum_f64(Cx<double>* out, const Geom* gp, const void* links, const void* in, int r,
-                                         int par, int cb, bool dagger) {
-  if (dagger) hop_sum_f64_t<true>(out, gp, links, in, r, par, cb);
-  else hop_sum_f64_t<false>(out, gp, links, in, r, par, cb);
+// the neighbour of s in direction mu (checkerboard index)
+__device__ __forceinline__ int fx_nbr(const Geom& g, const Site& s, int mu, bool bwd) {
+  const int c = mu & 2 ? (mu & 1 ? s.c[3] : s.c[2]) : (mu & 1 ? s.c[1] : s.c[0]);
+  const int L = g.L[mu], st = g.stride[mu];
+  return (bwd ? (c > 0 ? s.lex - st : s.lex + (L - 1) * st) : (c + 1 < L ? s.lex + st : s.lex - (L - 1) * st)) >> 1;
+}
+
+// The sums of a site in FP64 arithmetic, where the fixed point does not take it:
+// out[0..2] of spin sp and out[3..5] of spin 2 + sp, or only one of the two (rows 1: sp, 2:
+// 2 + sp, 3: both), by spin and pair of directions as in the kernel.  Not inlined: it is
+// rare.  Each warp of the site calls it for its own rows, so half hops are repeated: M of
+// a point source's solution, 16^3 x 32, 4 systems, takes 0.86 ms with links exp(0.3 i H)
+// and 1.43 with exp(0.1 i H), where almost every warp has such a site (FP64 kernel 0.81, without
+// such sites 0.24).  An exchange of the sums through shared memory takes 0.68 and 1.07, but
+// cost the solves 2%, by the registers and the code around it; the whole site in
+// each warp took 1.02 and 1.73.
+static __device__ __noinline__ void fx_sums_f64(Cx<double>* out, const DslashArgs* ap, int r, int par, int cb, int sp,
+                                                int rows) {
+  const DslashArgs& a = *ap;
+  const Geom& g = a.g;
+  const Site s = site_of(g, par, cb);
+  const int opar = par ^ 1, SF = a.c.dagger ? +1 : -1;
+  const size_t cs = (size_t)g.Vh;
+  Cx<double> u[3], l[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) u[c] = l[c] = {0.0, 0.0};
+  // spin sp over (x, y) and (z, t); over (x, y) the other upper spin, whose lower row is 2 + sp
+#pragma unroll 1
+  for (int k = 0; k < 3; ++k) {
+    if ((k == 0 && !(rows & 1)) || (k == 2 && !(rows & 2))) continue;
+    const int h = k == 2 ? sp ^ 1 : sp, it = k == 1;
+    const double2* fup = reinterpret_cast<const double2*>(a.c.in) + ((size_t)(r * 2 + opar) * 12 + 3 * h) * cs;
+    const double2* fdn = fup + (6 + 3 * (it ? 0 : 1 - 2 * h)) * (ptrdiff_t)cs;
+    const double2* uf = reinterpret_cast<const double2*>(a.links) + (size_t)(4 * it + par) * 9 * cs;  // next direction: + 18 cs
+    const double2* ub = reinterpret_cast<const double2*>(a.links) + (size_t)(4 * it + opar) * 9 * cs;
+    const int so = it && h ? -1 : 1, se = it || h ? 1 : -1;
+    const bool edge = it && g.antiperiodic;
+    Cx<double> up[3], lo[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) up[c] = lo[c] = {0.0, 0.0};
+    int n = fx_nbr(g, s, 2 * it, false);
+    f64_hop<true, false>(up, lo, fup + n, fdn + n, uf + cb, cs, SF * so, 1.0);
+    n = fx_nbr(g, s, 2 * it, true);
+    f64_hop<true, true>(up, lo, fup + n, fdn + n, ub + n, cs, -SF * so, 1.0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const Cx<double> v = lo[c];
+      lo[c] = so == se ? Cx<double>{v.im, -v.re} : Cx<double>{-v.im, v.re};
+    }
+    n = fx_nbr(g, s, 2 * it + 1, false);
+    f64_hop<false, false>(up, lo, fup + n, fdn + n, uf + 18 * cs + cb, cs, SF * se,
+                          edge && s.c[3] == g.L[3] - 1 ? -1.0 : 1.0);
+    n = fx_nbr(g, s, 2 * it + 1, true);
+    f64_hop<false, true>(up, lo, fup + n, fdn + n, ub + 18 * cs + n, cs, -SF * se, edge && s.c[3] == 0 ? -1.0 : 1.0);
+    const double f = se * SF;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      if (k < 2) u[c] = {__dadd_rn(u[c].re, up[c].re), __dadd_rn(u[c].im, up[c].im)};
+      if (k > 0) l[c] = {__fma_rn(f, lo[c].re, l[c].re), __fma_rn(f, lo[c].im, l[c].im)};
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    out[c] = u[c];
+    out[3 + c] = l[c];
+  }
 }
 
 // The FP64 epilogue (dslash_epilogue) of spin sp0 (acc[0..2]) and, with NC = 6,
@@ -297,17 +379,34 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp0, int 
   return NC == 6 ? __dadd_rn(part[0], part[1]) : part[0];
 }
 
+// Does a site need FP64 sums?  m: its (unit << 16 | least s of the rows, in units of
+// 2^-10 B) of [upper spin][pair of directions], E the common unit.  Spins that all
+// neighbours leave at zero are exact.
+__device__ __forceinline__ bool fx_small(const unsigned (&m)[2][2], unsigned E) {
+  constexpr unsigned kMin = 1024 / 4;
+  unsigned b[2][2];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) b[j >> 1][j & 1] = shr32(m[j >> 1][j & 1] & 0xffffu, E - (m[j >> 1][j & 1] >> 16));
+  bool small = false;
+#pragma unroll
+  for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+    for (int o = 0; o < 2; ++o)  // o = sp: spin sp; else spin 2 + sp, which takes (x, y) from the other upper spin
+      small = small || (b[o][0] + b[sp][1] < kMin && (m[o][0] | m[sp][1]) != 0);
+  return small;
+}
+
 // Two warps take 32 consecutive sites of one system, one for each upper spin
 // (with the lower rows it feeds), and exchange the lower row that belongs to
 // the other one through shared memory.  The loop over (x, y), (z, t) keeps 12
 // sums of 64 bits and the code small; the upper sums of (x, y) wait in shared
-// memory too.  The pairs of a block take 2^lgs systems
-// (fastest) of the same sites, whose links then come from L1, and the next
-// 32-site groups.
+// memory too.  The pairs of a block take 2^lgs systems (fastest) of the same sites,
+// whose links then come from L1, and the next 32-site groups.
 // The neighbours' words come by asynchronous copies to the lane's own slots in
 // shared memory, one hop ahead of the one computed: latency is covered without
 // registers (24^3 x 48, 12 systems, M: loads at their use 3.45 ms, copies 3.29;
-// FP64 arithmetic 12.2.  The same copies for the centre's words 3.40).  No fences
+// FP64 arithmetic 12.2; with a unit for each pair of directions and the sums S now 3.40.
+// The same copies for the centre's words another 3% longer).  No fences
 // or barriers: a lane reads what it copied, and a slot's words are in registers
 // before its next copy starts.
 // Bound by the integer multiplier (67% busy), fixed latencies of the 64-bit sums and
@@ -320,10 +419,11 @@ __device__ __forceinline__ double fx_epilogue(const DslashArgs& a, int sp0, int 
 // half the chain of a thread, for lattices that leave SMs idle (4^4, 16 systems:
 // 13.9 us, two warps 17.3, FP64 arithmetic 34.9).
 template <int EPI, bool QUAD>
-__global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const DslashArgs a, const int4* links_fx, int lgs) {
+__global__ void __launch_bounds__(128, QUAD ? 3 : 5)
+    dslash_fx_kernel(const __grid_constant__ DslashArgs a, const int4* links_fx, int lgs) {
   __shared__ FxStage ring[4][2];
   __shared__ longlong2 xu[4][3][32], xl[4][3][32];  // upper and lower sums on their way to another warp or loop
-  __shared__ unsigned xe[2][4][32];                 // units of [pair of warps][2 upper spin + pair of directions]
+  __shared__ unsigned meta[2][4][32];               // of [pair of warps][2 upper spin + pair of directions], see fx_small
   __shared__ double xsum[4];
   __shared__ double xpart[2][32];
   const Geom& g = a.g;
@@ -359,12 +459,7 @@ __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const Dsla
     const size_t cs = (size_t)g.Vh;
     const double2* fup = reinterpret_cast<const double2*>(a.c.in) + ((size_t)(r * 2 + opar) * 12 + 3 * sp) * cs;
     FxStage &s0 = ring[warp][0], &s1 = ring[warp][1];
-    // the neighbour in direction mu
-    auto nbr = [&](int mu, bool bwd) {
-      const int c = mu & 2 ? (mu & 1 ? s.c[3] : s.c[2]) : (mu & 1 ? s.c[1] : s.c[0]);
-      const int L = g.L[mu], st = g.stride[mu];
-      return (bwd ? (c > 0 ? s.lex - st : s.lex + (L - 1) * st) : (c + 1 < L ? s.lex + st : s.lex - (L - 1) * st)) >> 1;
-    };
+    auto nbr = [&](int mu, bool bwd) { return fx_nbr(g, s, mu, bwd); };
     // start the copy of neighbour n for a hop of pair it
     auto copy = [&](FxStage& st, int it, int n) {
       fx_copy(st, lane, fup + n, fup + (6 + 3 * (it ? 0 : 1 - 2 * sp)) * (ptrdiff_t)cs + n, cs);
@@ -380,6 +475,7 @@ __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const Dsla
       const bool ap = it && g.antiperiodic;
 #pragma unroll
       for (int c = 0; c < 3; ++c) t.upr[c] = t.upi[c] = t.lor[c] = t.loi[c] = 0;
+      t.s[0] = t.s[1] = t.s[2] = 0;
       t.E = kFxMinExp;
       t.big = 0;
       const int nb0 = nbr(2 * it, true);
@@ -418,7 +514,8 @@ __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const Dsla
         for (int c = 0; c < 3; ++c) xu[warp][c][lane] = make_longlong2(t.upr[c], t.upi[c]);
       }
       if ((t.big >> 20) > kFxMaxExp || (t.big != 0 && (t.big >> 20) < kFxMinExp)) t.E = kFxBad;
-      xe[pair][2 * sp + it][lane] = t.E;
+      if (t.big == 0) t.E = 0;
+      meta[pair][2 * sp + it][lane] = __byte_perm(min(min(t.s[0], t.s[1]), t.s[2]), t.E, 0x5432);
     }
   }
   __syncthreads();
@@ -429,24 +526,26 @@ __global__ void __launch_bounds__(128, QUAD ? 3 : 5) dslash_fx_kernel(const Dsla
     // other one spin 2 + sp with the lower ones of spin 1 - sp's (x, y)
     const int sp0 = QUAD && it0 ? 2 + sp : sp;
     Cx<double> acc[NC];
-    // the common unit of the site's sums; kFxBad if one of them is out of range
-    unsigned e[2][2];  // [this or the other upper spin][pair of directions]
+    // the common unit of the site's sums, the same in all its warps
+    unsigned m[2][2], e[2][2];  // [this or the other upper spin][pair of directions]
 #pragma unroll
-    for (int j = 0; j < 4; ++j) e[j >> 1][j & 1] = xe[pair][2 * (sp ^ (j >> 1)) + (j & 1)][lane];
-    const unsigned E = max(max(e[0][0], e[0][1]), max(e[1][0], e[1][1]));
-    double unit = __hiloint2double((int)(E - 55u) << 20, 0);  // 2^(E - 1078)
+    for (int j = 0; j < 4; ++j) {
+      m[j >> 1][j & 1] = meta[pair][2 * (sp ^ (j >> 1)) + (j & 1)][lane];
+      e[j >> 1][j & 1] = m[j >> 1][j & 1] >> 16;
+    }
+    unsigned E = max(max(e[0][0], e[0][1]), max(e[1][0], e[1][1]));
+    if (fx_small(m, E)) E = kFxBad;
+    E = max(E, kFxMinExp);
+    double unit = __hiloint2double((int)(E - 56u) << 20, 0);  // 2^(E - 1079)
     if (E == kFxBad) {
-      Cx<double> all[12];
-      hop_sum_f64(all, &a.g, a.links, a.c.in, r, par, cb, a.c.dagger);
+      Cx<double> f[6];
+      fx_sums_f64(f, &a, r, par, cb, sp, QUAD ? 1 + it0 : 3);
 #pragma unroll
-      for (int q = 0; q < NC; ++q) {
-        const int c = q % 3;
-        const Cx<double> u = sp == 0 ? all[c] : all[3 + c], l = sp == 0 ? all[6 + c] : all[9 + c];
-        acc[q] = (QUAD ? it0 != 0 : q >= 3) ? l : u;
-      }
+      for (int q = 0; q < NC; ++q) acc[q] = f[QUAD && it0 ? 3 + q : q];
       unit = 1.0;
     } else {
-      const unsigned d0 = E - e[0][0], d1 = E - e[0][1], dx = E - e[1][0];
+      // one more bit: the sums of four hops may fill 63
+      const unsigned d0 = E - e[0][0] + 1, d1 = E - e[0][1] + 1, dx = E - e[1][0] + 1;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         if (!QUAD || it0 == 0) {

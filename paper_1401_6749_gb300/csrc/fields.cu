@@ -257,48 +257,75 @@ __global__ void pack_links_kernel(Geom g, void* out, const double* U) {
 }
 
 // canonical FP64 links -> fixed-point halves [mu][parity][group of 32 sites][9][32]: a part u as
-// round(u 2^54) = hi 2^27 + lo, |lo| <= 2^26, one complex number per 16 bytes
-// (re.hi, re.lo, im.hi, im.lo); *bad is set if a part exceeds 1.25 or is not
-// a number
-__device__ __forceinline__ int2 fx_link(double u, bool& bad) {
-  if (!(fabs(u) <= 1.25)) {
-    bad = true;
-    return make_int2(0, 0);
-  }
-  const long long q = __double2ll_rn(u * 18014398509481984.0);  // 2^54
-  const int lo = (int)((q + (1 << 26)) & ((1 << 27) - 1)) - (1 << 26);
-  return make_int2((int)((q - lo) >> 27), lo);
+// round(u 2^58) = hi 2^29 + lo, |lo| <= 2^28, one complex number per 16 bytes
+// (re.hi, re.lo, im.hi, im.lo).  stat[0] is set if a row or column has a norm above
+// 1.5 or a part is not a number; stat[1] and stat[2] are the sums of max(|re|, |im|) and
+// min(|re|, |im|) over all entries, in units of 2^-10 (integers: in any order the same).
+__device__ __forceinline__ int2 fx_link(double u) {
+  const long long q = __double2ll_rn(u * 288230376151711744.0);  // 2^58
+  const int lo = (int)((q + (1 << 28)) & ((1 << 29) - 1)) - (1 << 28);
+  return make_int2((int)((q - lo) >> 29), lo);
 }
 
-__global__ void pack_links_fx_kernel(Geom g, int4* out, const double* U, int* bad) {
+__global__ void __launch_bounds__(256) pack_links_fx_kernel(Geom g, int4* out, const double* U,
+                                                            unsigned long long* stat) {
   const long V = 2L * g.Vh;
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 4 * V) return;
-  const int mu = (int)(i / V);
-  const int lex = (int)(i % V);
-  const int x = lex % g.L[0], y = (lex / g.stride[1]) % g.L[1];
-  const int z = (lex / g.stride[2]) % g.L[2], t = lex / g.stride[3];
-  const int par = (x + y + z + t) & 1;
-  const double2* src = reinterpret_cast<const double2*>(U) + ((size_t)mu * V + lex) * 9;
-  const size_t cb = (size_t)(lex >> 1), nw = (size_t)((g.Vh + 31) >> 5);
-  int4* dst = out + ((size_t)(mu * 2 + par) * nw + (cb >> 5)) * 288 + (cb & 31);
-  bool b = false;
+  unsigned big = 0, small = 0;
+  bool ok = true;
+  if (i < 4 * V) {
+    const int mu = (int)(i / V);
+    const int lex = (int)(i % V);
+    const int x = lex % g.L[0], y = (lex / g.stride[1]) % g.L[1];
+    const int z = (lex / g.stride[2]) % g.L[2], t = lex / g.stride[3];
+    const int par = (x + y + z + t) & 1;
+    const double2* src = reinterpret_cast<const double2*>(U) + ((size_t)mu * V + lex) * 9;
+    const size_t cb = (size_t)(lex >> 1), nw = (size_t)((g.Vh + 31) >> 5);
+    int4* dst = out + ((size_t)(mu * 2 + par) * nw + (cb >> 5)) * 288 + (cb & 31);
+    double norm[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // squares, of rows and columns
 #pragma unroll
-  for (int u = 0; u < 9; ++u) {
-    const double2 v = src[u];
-    const int2 re = fx_link(v.x, b), im = fx_link(v.y, b);
-    dst[u * 32] = make_int4(re.x, re.y, im.x, im.y);
+    for (int u = 0; u < 9; ++u) {
+      const double2 v = src[u];
+      const double n = v.x * v.x + v.y * v.y;
+      norm[u / 3] += n;
+      norm[3 + u % 3] += n;
+      big += __double2uint_rn(1024.0 * fmax(fabs(v.x), fabs(v.y)));
+      small += __double2uint_rn(1024.0 * fmin(fabs(v.x), fabs(v.y)));
+      const int2 re = fx_link(v.x), im = fx_link(v.y);
+      dst[u * 32] = make_int4(re.x, re.y, im.x, im.y);
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) ok = ok && norm[k] <= 2.25;  // false for NaN
   }
-  if (b) atomicOr(bad, 1);
+  const bool all = __syncthreads_and(ok);
+  __shared__ unsigned sum[2];
+  if (threadIdx.x < 2) sum[threadIdx.x] = 0;
+  __syncthreads();
+  big = __reduce_add_sync(0xffffffffu, big);
+  small = __reduce_add_sync(0xffffffffu, small);
+  if (threadIdx.x % 32 == 0) {
+    atomicAdd(&sum[0], big);
+    atomicAdd(&sum[1], small);
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) atomicAdd(stat + 1 + threadIdx.x, (unsigned long long)sum[threadIdx.x]);
+  if (threadIdx.x == 0 && !all) atomicOr(stat, 1ull);
 }
 
 size_t links_fx_bytes(const Geom& g) { return 8 * (size_t)nwarp_of(g) * 288 * sizeof(int4); }
 
-tm_status_t pack_links_fx(const Geom& g, void* out, const double* U, int* bad, cudaStream_t s) {
-  pack_links_fx_kernel<<<blocks_for(4L * 2 * g.Vh, 256), 256, 0, s>>>(g, static_cast<int4*>(out), U, bad);
+tm_status_t pack_links_fx(const Geom& g, void* out, const double* U, unsigned long long* stat, cudaStream_t s) {
+  pack_links_fx_kernel<<<blocks_for(4L * 2 * g.Vh, 256), 256, 0, s>>>(g, static_cast<int4*>(out), U, stat);
   count_launch();
   return check_launch("pack_links_fx");
 }
+
+// Does the fixed point take these links?  Its errors are bounded against complex numbers
+// w = W h (dslash_fx.cuh).  Real and imaginary parts that differ in size have to mix in
+// the links for that to hold of each of them: not so for unit or real links.  exp(i eps H)
+// has a quotient of the sums of 0.04 at eps = 0.05, 0.08 at 0.1, 0.21 at 0.3.  Links below the
+// line take the FP64 kernel.
+bool links_fx_ok(const unsigned long long* stat) { return stat[0] == 0 && 16 * stat[2] >= stat[1]; }
 
 template <class S, int RECON>
 static size_t link_bytes_t(const Geom& g) {

@@ -34,8 +34,8 @@ struct tm_op {
   int recon_p[tml::kNumPrec];  // link format (12 or 18 reals) of the copy of each precision
   void* links[tml::kNumPrec];  // indexed by tm_prec_t; F64 and FF always 18-real
   // FP64 links as fixed-point halves for the FP64 Dslash (dslash_fx.cuh),
-  // [mu][parity][group of 32 sites][9][32] x 16 bytes; null if a link has a
-  // component beyond 1.25
+  // [mu][parity][group of 32 sites][9][32] x 16 bytes; null if it does not take these
+  // links (links_fx_ok, fields.cu)
   void* links_fx;
   // solver work space, grown on demand, owned by the operator
   void* work;
