@@ -68,10 +68,9 @@ __device__ __forceinline__ Cx<R> mom_phase(const Geom& g, const Mom3& q, const S
   }
 }
 
-// MOM: the site's R is multiplied by exp(-i p.x) (a single non-zero momentum)
-template <class S, bool MOM = false>
+template <class S>
 __global__ void __launch_bounds__(256) local_partial_kernel(Geom g, const void* Lf, const void* Rf,
-                                                            int nchunk, double* partial, Mom3 mom = Mom3{}) {
+                                                            int nchunk, double* partial) {
   using R = typename Prec<S>::R;
   const int chunk = (int)blockIdx.x;
   const int t = blockIdx.y >> 1, par = blockIdx.y & 1;
@@ -87,11 +86,6 @@ __global__ void __launch_bounds__(256) local_partial_kernel(Geom g, const void* 
       Cx<R> l[12], r[12];
       load_spinor<S>(l, Lf, b0, (size_t)g.Vh);
       load_spinor<S>(r, Rf, b0, (size_t)g.Vh);
-      if constexpr (MOM) {
-        const Cx<R> ph = mom_phase<R>(g, mom, site_of(g, par, t * g.V3h + i));
-#pragma unroll
-        for (int k = 0; k < 12; ++k) r[k] = ph * r[k];
-      }
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -147,29 +141,38 @@ __global__ void mom_phase_kernel(Geom g, MomList mom, int q0, int nq, Cx<R>* ph)
 // over eight sites and are then added with compensation (two-sum), so their
 // error stays that of a short sum.  Bound by the FMA pipe (64 FMAs per site and
 // momentum); a pass per momentum, which it replaces, formed the 16 bilinears
-// and the phase again for each.
+// and the phase again for each.  QT = 0: one momentum; the lane groups take its
+// terms of eight sites in turn and these are added in the order of the other
+// forms, so that a momentum's bits do not depend on the list it is asked in.
 constexpr int kMomTile = 128;
+__device__ __forceinline__ FF shfl_from(FF v, int l) {
+  return {__shfl_sync(0xffffffffu, v.hi, l), __shfl_sync(0xffffffffu, v.lo, l)};
+}
+template <class R>
+__device__ __forceinline__ R shfl_from(R v, int l) { return __shfl_sync(0xffffffffu, v, l); }
 template <class S, int QT>
-__global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const void* Lf, const void* Rf, int nchunk,
-                                                               const void* phases, int q0, int nmom, double* partial) {
+__global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const void* Lf, const void* Rf, int nsite,
+                                                               int nchunk, const void* phases, MomList mom, int q0,
+                                                               double* partial) {
   using R = typename Prec<S>::R;
   using O = Ar<R>;
   extern __shared__ __align__(16) unsigned char mom_smem[];
   Cx<R>* sm = reinterpret_cast<Cx<R>*>(mom_smem);  // [site][8 pairs, swizzled by site][2]
-  Cx<R>* sp = sm + kMomTile * 16;                  // [site][4 QT]
-  constexpr int nq = 4 * QT;
+  Cx<R>* sp = sm + kMomTile * 16;                  // [site][nq]
+  constexpr bool ONE = QT == 0;
+  constexpr int nq = ONE ? 1 : 4 * QT, NA = ONE ? 1 : QT;  // momenta of the pass and of a lane
   const int chunk = (int)blockIdx.x;
   const int t = blockIdx.y >> 1, par = blockIdx.y & 1;
   const int rhs = blockIdx.z;
   const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
   const int cg = lane & 7, qg = lane >> 3;
   const Cx<R>* ph = static_cast<const Cx<R>*>(phases) + (size_t)((t + par) & 1) * g.V3h * nq;
-  Cx<R> acc[QT][2], err[QT][2];
+  Cx<R> acc[NA][2], err[NA][2];
 #pragma unroll
-  for (int j = 0; j < QT; ++j) acc[j][0] = acc[j][1] = err[j][0] = err[j][1] = {(R)0, (R)0};
-  const int iend = min(g.V3h, (chunk + 1) * kLocalChunk);
+  for (int j = 0; j < NA; ++j) acc[j][0] = acc[j][1] = err[j][0] = err[j][1] = {(R)0, (R)0};
+  const int iend = min(g.V3h, (chunk + 1) * nsite);
 #pragma unroll 1
-  for (int i0 = chunk * kLocalChunk; i0 < iend; i0 += kMomTile) {
+  for (int i0 = chunk * nsite; i0 < iend; i0 += kMomTile) {
     const int i = i0 + (int)threadIdx.x;
     Cx<R> m[16];
 #pragma unroll
@@ -199,21 +202,30 @@ __global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const voi
 #pragma unroll
     for (int k = 0; k < 16; ++k) sm[threadIdx.x * 16 + 2 * ((k >> 1) ^ (threadIdx.x & 7)) + (k & 1)] = m[k];
     const int rows = min(kMomTile, iend - i0);
-    for (int k = threadIdx.x; k < rows * nq; k += kMomTile) sp[k] = ph[(size_t)i0 * nq + k];
-    __syncthreads();
+    if (QT > 1 || phases) {
+      for (int k = threadIdx.x; k < rows * nq; k += kMomTile) sp[k] = ph[(size_t)i0 * nq + k];
+    } else if ((int)threadIdx.x < rows) {
+      const Site st = site_of(g, par, t * g.V3h + i);
 #pragma unroll 1
-    for (int s0 = wq; s0 < rows; s0 += 32) {
-      Cx<R> z[QT][2];
+      for (int q = 0; q < nq && q0 + q < mom.n; ++q) sp[threadIdx.x * nq + q] = mom_phase<R>(g, mom.q[q0 + q], st);
+#pragma unroll 1
+      for (int q = max(0, mom.n - q0); q < nq; ++q) sp[threadIdx.x * nq + q] = {(R)0, (R)0};
+    }
+    __syncthreads();
+    // one momentum: each lane group takes 32 sites of the warp's, and all add them in order
+#pragma unroll 1
+    for (int s0 = ONE ? wq + 32 * qg : wq; s0 < (ONE ? wq + 32 * qg + 1 : rows); s0 += 32) {
+      Cx<R> z[NA][2];
 #pragma unroll
-      for (int j = 0; j < QT; ++j) z[j][0] = z[j][1] = {(R)0, (R)0};
+      for (int j = 0; j < NA; ++j) z[j][0] = z[j][1] = {(R)0, (R)0};
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const int s = s0 + 4 * k;
         if (s < rows) {
           const Cx<R> m0 = sm[s * 16 + 2 * (cg ^ (s & 7))], m1 = sm[s * 16 + 2 * (cg ^ (s & 7)) + 1];
 #pragma unroll
-          for (int j = 0; j < QT; ++j) {
-            const Cx<R> p = sp[s * nq + qg * QT + j];
+          for (int j = 0; j < NA; ++j) {
+            const Cx<R> p = sp[s * nq + (ONE ? 0 : qg * QT + j)];
             z[j][0] = {O::fma(-p.im, m0.im, O::fma(p.re, m0.re, z[j][0].re)), O::fma(p.im, m0.re, O::fma(p.re, m0.im, z[j][0].im))};
             z[j][1] = {O::fma(-p.im, m1.im, O::fma(p.re, m1.re, z[j][1].re)), O::fma(p.im, m1.re, O::fma(p.re, m1.im, z[j][1].im))};
           }
@@ -229,62 +241,94 @@ __global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const voi
         }
       };
 #pragma unroll
-      for (int j = 0; j < QT; ++j)
+      for (int g0 = 0; g0 < (ONE ? 4 : 1); ++g0) {
+        if (ONE && wq + 32 * g0 >= rows) break;
+        auto from = [&](R v) { return ONE ? shfl_from(v, 8 * g0 + cg) : v; };
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          add(acc[j][c].re, err[j][c].re, z[j][c].re);
-          add(acc[j][c].im, err[j][c].im, z[j][c].im);
-        }
+        for (int j = 0; j < NA; ++j)
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            add(acc[j][c].re, err[j][c].re, from(z[j][c].re));
+            add(acc[j][c].im, err[j][c].im, from(z[j][c].im));
+          }
+      }
     }
   }
   // the warps' sums, in order, in FP64
   __syncthreads();
   double* red = reinterpret_cast<double*>(mom_smem);  // [warp][q of the group][32]
   static_assert(sizeof(double) * 4 * 32 * nq <= sizeof(Cx<R>) * kMomTile * (16 + nq), "the sums fit the tiles");
+  if (!ONE || qg == 0) {
 #pragma unroll
-  for (int j = 0; j < QT; ++j)
+    for (int j = 0; j < NA; ++j)
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      double* w = red + ((size_t)wq * nq + qg * QT + j) * 32 + 2 * (2 * cg + c);
-      w[0] = (double)acc[j][c].re + (double)err[j][c].re;
-      w[1] = (double)acc[j][c].im + (double)err[j][c].im;
-    }
+      for (int c = 0; c < 2; ++c) {
+        double* w = red + ((size_t)wq * nq + qg * QT + j) * 32 + 2 * (2 * cg + c);
+        w[0] = (double)acc[j][c].re + (double)err[j][c].re;
+        w[1] = (double)acc[j][c].im + (double)err[j][c].im;
+      }
+  }
   __syncthreads();
   for (int k = threadIdx.x; k < nq * 32; k += kMomTile) {
     const int q = q0 + (k >> 5);
-    if (q >= nmom) continue;
+    if (q >= mom.n) continue;
     double v = 0.0;
 #pragma unroll
     for (int w = 0; w < 4; ++w) v += red[(size_t)w * nq * 32 + k];
-    const size_t slot = ((((size_t)rhs * nmom + q) * g.L[3] + t) * 2 + par) * nchunk + chunk;
+    const size_t slot = ((((size_t)rhs * mom.n + q) * g.L[3] + t) * 2 + par) * nchunk + chunk;
     partial[slot * 32 + (k & 31)] = v;
   }
 }
 
-// at most 32 momenta per pass: QT momenta per lane group
+// at most 32 momenta per pass: QT momenta per lane group, 0 for a single one.  4 and 6 are
+// left out to keep the code small (a form is five kernels): they would save
+// lists of 13 to 16 and of 21 to 24 momenta a fifth and a seventh of the FMAs.
 constexpr int kMomPass = 32;
+static int mom_nq(int qt) { return qt == 0 ? 1 : 4 * qt; }
 static int mom_qt(int nq) {
+  if (nq == 1) return 0;
   const int q = (nq + 3) / 4;
   return q <= 1 ? 1 : q <= 2 ? 2 : q <= 3 ? 3 : q <= 5 ? 5 : q <= 7 ? 7 : 8;
 }
 
+// Sites per block: 1024, or fewer where one system would leave SMs without a block;
+// by the lattice alone, for they set the order of the sums.  Two momenta, FP32, one system,
+// 16^3 x 32: 29 us with 512 (the rule), 37 with 1024, 25 with 256, which costs 16 systems
+// and 19 momenta 353 us against 303; float-float, 19 momenta, 8^3 x 16: 56 us against 82.
+static int mom_sites(const Geom& g) {
+  int n = kLocalChunk;
+  while (n > kMomTile && 2 * g.L[3] * ((g.V3h + n - 1) / n) < 256) n /= 2;
+  return n;
+}
+// A table of phases, or each block makes its own (up to four momenta: a thread makes its
+// site's one after the other).  Its own are faster where there are few, by about the launch of
+// the table: 8^3 x 16, one system, one and two momenta, FP32: 22 against 24 us, float-float 23.3 and
+// 25.4 against 26.0 and 27.6; slower from 2^17 phases on (16^3 x 32, one momentum, float-float, one
+// system: 57 against 47; 4 systems, FP32: 54 against 42).
+static bool mom_table(const Geom& g, int nrhs, int nq) { return nq > 4 || 2.0 * g.Vh * nrhs * nq > 65536.0; }
+
 template <class S, int QT>
 static tm_status_t mom_launch(const Geom& g, const void* left, const void* right, int nrhs, const MomList& ml, int q0,
-                              void* phases, int nchunk, double* scratch, cudaStream_t s) {
+                              void* phases, int nsite, double* scratch, cudaStream_t s) {
   using R = typename Prec<S>::R;
-  constexpr int nq = 4 * QT, smem = (int)sizeof(Cx<R>) * kMomTile * (16 + nq);
+  constexpr int nq = QT == 0 ? 1 : 4 * QT, smem = (int)sizeof(Cx<R>) * kMomTile * (16 + nq);
   if (smem > 48 * 1024 &&
       cudaFuncSetAttribute(mom_partial_kernel<S, QT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
           cudaSuccess) {
     set_error("loop_contract_local_mom: %s", cudaGetErrorString(cudaGetLastError()));
     return TM_ERR_CUDA;
   }
-  const long np = 2L * g.V3h * nq;
-  mom_phase_kernel<R><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(g, ml, q0, nq, static_cast<Cx<R>*>(phases));
-  count_launch();
-  TM_TRY(check_launch("loop_contract_local_mom phases"));
+  if (mom_table(g, nrhs, nq)) {
+    const long np = 2L * g.V3h * nq;
+    mom_phase_kernel<R><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(g, ml, q0, nq, static_cast<Cx<R>*>(phases));
+    count_launch();
+    TM_TRY(check_launch("loop_contract_local_mom phases"));
+  } else {
+    phases = nullptr;
+  }
+  const int nchunk = (g.V3h + nsite - 1) / nsite;
   const dim3 grid(nchunk, 2 * g.L[3], nrhs);
-  mom_partial_kernel<S, QT><<<grid, kMomTile, smem, s>>>(g, left, right, nchunk, phases, q0, ml.n, scratch);
+  mom_partial_kernel<S, QT><<<grid, kMomTile, smem, s>>>(g, left, right, nsite, nchunk, phases, ml, q0, scratch);
   count_launch();
   return check_launch("loop_contract_local_mom");
 }
@@ -849,12 +893,12 @@ extern "C" tm_status_t loop_contract_local_mom(const tm_geom_t* gg, const void* 
       ml.q[q].p[k] = ((mom[3 * q + k] % Lk) + Lk) % Lk;  // p and p + L are the same momentum
     }
   const int n2 = nrhs * n_mom;
-  const int nchunk = (g.V3h + kLocalChunk - 1) / kLocalChunk;
-  // several momenta: the table of phases of one pass behind the partial sums
-  const size_t part = local_scratch_bytes(g, n2), cplx = prec == TM_PREC_F64 || prec == TM_PREC_FF ? 16 : 8;
-  const int nq_max = 4 * mom_qt(n_mom < kMomPass ? n_mom : kMomPass);
+  const int nsite = mom_sites(g), nchunk = (g.V3h + nsite - 1) / nsite;
+  // the table of phases of one pass behind the partial sums
+  const size_t part = sizeof(double) * 32 * (size_t)n2 * g.L[3] * 2 * nchunk, cplx = prec == TM_PREC_F64 || prec == TM_PREC_FF ? 16 : 8;
+  const int nq_max = mom_nq(mom_qt(n_mom < kMomPass ? n_mom : kMomPass));
   double* scratch = nullptr;
-  tm_status_t st = scratch_alloc((void**)&scratch, part + (n_mom > 1 ? 2 * (size_t)g.V3h * nq_max * cplx : 0), s);
+  tm_status_t st = scratch_alloc((void**)&scratch, part + 2 * (size_t)g.V3h * nq_max * cplx, s);
   if (st != TM_OK) return st;
   void* phases = reinterpret_cast<char*>(scratch) + part;
   {
@@ -863,27 +907,16 @@ extern "C" tm_status_t loop_contract_local_mom(const tm_geom_t* gg, const void* 
     TraceScope tr(s, prec_name(kNames, prec), 2.0 * 24.0 * prec_size(prec) * 2.0 * g.Vh, 0.0, n2);
     st = by_prec_c(prec, [&](auto tag) {
       using S = decltype(tag);
-      if (n_mom == 1) {
-        // one momentum needs no table: 404 us at 24^3 x 48, FP32, 12 systems, against
-        // 434 us by the table and the matrix product; zero momentum, no phase
-        const dim3 grid(nchunk, 2 * g.L[3], nrhs);
-        const Mom3& q = ml.q[0];
-        if (q.p[0] || q.p[1] || q.p[2])
-          local_partial_kernel<S, true><<<grid, 256, 0, s>>>(g, left, right, nchunk, scratch, q);
-        else
-          local_partial_kernel<S><<<grid, 256, 0, s>>>(g, left, right, nchunk, scratch);
-        count_launch();
-        return check_launch("loop_contract_local_mom");
-      }
       for (int q0 = 0; q0 < n_mom; q0 += kMomPass) {
         tm_status_t ps;
         switch (mom_qt(n_mom - q0 < kMomPass ? n_mom - q0 : kMomPass)) {
-          case 1: ps = mom_launch<S, 1>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s); break;
-          case 2: ps = mom_launch<S, 2>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s); break;
-          case 3: ps = mom_launch<S, 3>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s); break;
-          case 5: ps = mom_launch<S, 5>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s); break;
-          case 7: ps = mom_launch<S, 7>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s); break;
-          default: ps = mom_launch<S, 8>(g, left, right, nrhs, ml, q0, phases, nchunk, scratch, s); break;
+          case 0: ps = mom_launch<S, 0>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
+          case 1: ps = mom_launch<S, 1>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
+          case 2: ps = mom_launch<S, 2>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
+          case 3: ps = mom_launch<S, 3>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
+          case 5: ps = mom_launch<S, 5>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
+          case 7: ps = mom_launch<S, 7>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
+          default: ps = mom_launch<S, 8>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
         }
         if (ps != TM_OK) return ps;
       }

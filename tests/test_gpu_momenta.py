@@ -1,6 +1,6 @@
 """Momentum-projected local loops, all momenta of a pass in one kernel: at the
 edges of the momentum groups (4, 8, ..., 32 per pass) and of the site tiles (128)
-and chunks (1024), against the FP64 oracle.
+and chunks (128 to 1024), against the FP64 oracle.
 
 Tolerance: an output sums 4 phased bilinears per site.  In FP32 a bilinear of
 three complex products errs by at most 7 u sum_c |L||R|, its phase by 4 u, a sum of
@@ -59,3 +59,23 @@ def test_wide_full_pass(prec):
 @pytest.mark.parametrize("prec", ["f16", "f32", "ff", "f64"])
 def test_single_momentum(p, prec):
     _check((8, 6, 4, 6), 2, 1, prec, "vv", np.array([p]))
+
+
+@pytest.mark.parametrize("prec", ["f16", "f32", "ff", "f64"])
+@pytest.mark.parametrize("L", [(8, 6, 4, 6), (16, 12, 12, 2), (10, 10, 14, 2)])
+def test_list_independence(L, prec):
+    """A momentum alone and in a list: the same bits."""
+    tl = require_gpu()
+    p, n = tl.PREC[prec], 2
+    fl, fr = (pack(tl, L, synth.random_spinor(L, n, s), p) for s in (4, 5))
+
+    def loops(mom):
+        out = torch.full((n, len(mom), 16, L[3], 2), float("nan"), dtype=torch.float64, device="cuda")
+        tl.loop_contract_local_mom(L, fl, fr, p, n, tl.LOOP_MODE["vv"], mom, out)
+        return out
+
+    mom = _momenta(34)
+    many = loops(mom)
+    for k in (0, 1, 32, 33):
+        assert torch.equal(loops(mom[k:k + 1])[:, 0], many[:, k])
+    assert torch.equal(loops(mom[:5]), many[:, :5])
