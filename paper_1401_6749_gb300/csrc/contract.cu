@@ -904,7 +904,14 @@ extern "C" tm_status_t loop_contract_local_mom(const tm_geom_t* gg, const void* 
   {
     static const char* const kNames[kNumPrec] = {"localmom.f64", "localmom.f32", "localmom.f16", "localmom.bf16",
                                                   "localmom.ff"};
-    TraceScope tr(s, prec_name(kNames, prec), 2.0 * 24.0 * prec_size(prec) * 2.0 * g.Vh, 0.0, n2);
+    // per pass both fields once, and the table of phases written and read
+    double tables = 0.0;
+    int passes = 0;
+    for (int q0 = 0; q0 < n_mom; q0 += kMomPass, ++passes) {
+      const int nq = mom_nq(mom_qt(n_mom - q0 < kMomPass ? n_mom - q0 : kMomPass));
+      if (mom_table(g, nrhs, nq)) tables += 2.0 * 2.0 * g.V3h * nq * (double)cplx;
+    }
+    TraceScope tr(s, prec_name(kNames, prec), passes * 2.0 * 24.0 * prec_size(prec) * 2.0 * g.Vh, tables, nrhs);
     st = by_prec_c(prec, [&](auto tag) {
       using S = decltype(tag);
       for (int q0 = 0; q0 < n_mom; q0 += kMomPass) {

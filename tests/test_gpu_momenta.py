@@ -79,3 +79,25 @@ def test_list_independence(L, prec):
     for k in (0, 1, 32, 33):
         assert torch.equal(loops(mom[k:k + 1])[:, 0], many[:, k])
     assert torch.equal(loops(mom[:5]), many[:, :5])
+
+
+@pytest.mark.parametrize("nmom", [1, 4, 19, 32, 33])
+def test_trace_bytes(nmom):
+    """The record charges both fields once per pass of at most 32 momenta, and a
+    small part more for the phases; not once per momentum."""
+    tl = require_gpu()
+    L, n = (8, 8, 8, 16), 3
+    fields = 2 * n * 24 * 4 * int(np.prod(L))
+    fl, fr = (pack(tl, L, synth.random_spinor(L, n, s), tl.F32) for s in (4, 5))
+    out = torch.empty((n, nmom, 16, L[3], 2), dtype=torch.float64, device="cuda")
+    tl.tm_trace_reset()
+    tl.tm_trace_enable(True)
+    try:
+        tl.loop_contract_local_mom(L, fl, fr, tl.F32, n, tl.LOOP_MODE["vv"], _momenta(nmom), out)
+        launches, _, nbytes = tl.tm_trace_read("localmom.f32")
+    finally:
+        tl.tm_trace_enable(False)
+        tl.tm_trace_reset()
+    passes = (nmom + 31) // 32
+    assert launches == 1
+    assert passes * fields <= nbytes <= 1.2 * passes * fields
