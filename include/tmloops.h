@@ -96,7 +96,12 @@ typedef struct tm_op tm_op_t;
 
 /* Create an operator: validates p, copies the FP64 canonical gauge field
  * U_lex ([4][V][3][3][2] doubles, not retained) into internal even/odd link
- * arrays for every precision.  U_lex is device memory, or page-locked host
+ * arrays for every precision.  The F64 links are kept in a second form too, 64-bit
+ * fixed point (as many bytes again, 576 per site), on which the F64 Dslash runs several
+ * times as fast; not if the links mix real and imaginary parts too little (unit
+ * links), have a row or column of norm above 1.5, or if there is no memory for
+ * it.  Either way an F64 result has the accuracy of FP64 arithmetic, relative to the
+ * terms that each component sums, and a system's bits do not depend on the others.  U_lex is device memory, or page-locked host
  * memory (cudaHostAlloc / cudaHostRegister, 16-byte aligned) that the GPU reads
  * in one pass of its SMs over the host link into a staging buffer; other host
  * memory is TM_ERR_ARG.  Blocks until done.                               */

@@ -525,23 +525,24 @@ extern "C" tm_status_t tm_op_create(tm_op_t** out, const tm_params_t* p, const d
       }
     }
   }
-  // fixed-point copy for the FP64 Dslash, and whether it takes these links
+  // fixed-point copy for the FP64 Dslash, and whether it takes these links.  Without
+  // the memory for it the FP64 kernel on the copy above does the work.
   unsigned long long* fx_stat = nullptr;
   unsigned long long h_stat[3] = {0, 0, 0};
-  {
-    tm_status_t s5 = dev_alloc(&op->links_fx, links_fx_bytes(op->g), st, "tm_op_create");
-    if (s5 == TM_OK) s5 = dev_alloc((void**)&fx_stat, sizeof(h_stat), st, "tm_op_create");
-    if (s5 == TM_OK && cudaMemsetAsync(fx_stat, 0, sizeof(h_stat), st) != cudaSuccess) s5 = TM_ERR_CUDA;
-    if (s5 == TM_OK) s5 = pack_links_fx(op->g, op->links_fx, U, fx_stat, st);
-    if (s5 == TM_OK && cudaMemcpyAsync(h_stat, fx_stat, sizeof(h_stat), cudaMemcpyDeviceToHost, st) != cudaSuccess)
-      s5 = TM_ERR_CUDA;
+  if (dev_alloc(&op->links_fx, links_fx_bytes(op->g), st, "tm_op_create") == TM_OK &&
+      dev_alloc((void**)&fx_stat, sizeof(h_stat), st, "tm_op_create") == TM_OK) {
+    cudaError_t ce = cudaMemsetAsync(fx_stat, 0, sizeof(h_stat), st);
+    const tm_status_t s5 = ce == cudaSuccess ? pack_links_fx(op->g, op->links_fx, U, fx_stat, st) : TM_ERR_CUDA;
+    if (s5 == TM_OK) ce = cudaMemcpyAsync(h_stat, fx_stat, sizeof(h_stat), cudaMemcpyDeviceToHost, st);
     dev_free(fx_stat, st);
-    if (s5 != TM_OK) {
-      if (s5 == TM_ERR_CUDA) cudaGetLastError();
+    if (ce != cudaSuccess) set_error("tm_op_create: %s", cudaGetErrorString(cudaGetLastError()));
+    if (s5 != TM_OK || ce != cudaSuccess) {
       dev_free(staged, st);
       tm_op_destroy(op);
-      return s5;
+      return TM_ERR_CUDA;
     }
+  } else {
+    h_stat[0] = 1;
   }
   dev_free(staged, st);  // stream-ordered: after the packing that reads it
   if (op->il_err) {
