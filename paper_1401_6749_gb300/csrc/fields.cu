@@ -362,15 +362,12 @@ tm_status_t pack_links(const Geom& g, tm_prec_t p, int recon, void* out, const d
 }
 
 // ------------------------------------------------------------ solver BLAS
-// v 2^k by an integer addition on the exponent, in place of a multiplication on
-// the FP64 pipe: exact in the normal range; denormal results and arguments become
-// zero and results beyond the range infinite (infinities and NaN stay)
+// v 2^k, by an integer addition on the exponent in place of a multiplication on the
+// FP64 pipe where v and the result are normal
 __device__ __forceinline__ double mul_pow2(double v, int k) {
   const int h = __double2hiint(v), e = (h >> 20) & 0x7ff, n = e + k;
-  const bool zero = e == 0 || (n <= 0 && e != 0x7ff), inf = n >= 0x7ff && e != 0x7ff && e != 0;
-  const int m = h + (e != 0x7ff ? k << 20 : 0);
-  const int sign = h & (int)0x80000000;
-  return __hiloint2double(zero ? sign : inf ? sign | 0x7ff00000 : m, zero || inf ? 0 : __double2loint(v));
+  if (e > 0 && e < 0x7ff && n > 0 && n < 0x7ff) return __hiloint2double(h + k * (1 << 20), __double2loint(v));
+  return v == 0.0 ? v : scalbn(v, k);
 }
 
 // p = r + beta[rhs] p for active systems.  In mixed solves (r64 != null, stored as

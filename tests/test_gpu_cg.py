@@ -198,3 +198,20 @@ def test_schur_needs_fewer_iterations_and_is_batch_independent():
     tl.tm_cg_solve(op, xb, pack(tl, L, eta[4:5], 2), 1, lp)
     np.testing.assert_array_equal(unpack(tl, L, xa, 2, 6)[4], unpack(tl, L, xb, 2, 1)[0])
     op.close()
+
+
+def test_mixed_keeps_denormal_components():
+    """The rescaled residual keeps components below the normal range of FP64: with
+    unit links the colours are separate systems under the same polynomial, so a
+    colour of 2^-1030 times the source of another has as much of its solution."""
+    tl = require_gpu()
+    L, n = (4, 4, 4, 8), 1
+    op = tl.Operator(L, 0.12, 0.05, to_dev(synth.unit_gauge(L)), recon=18)
+    eta = oracle_z4(L, 5, 0, n)
+    eta[..., 2] = 2.0 ** -1000 * eta[..., 0] * 2.0 ** -30
+    x = tl.empty_field(L, 0, n)
+    tl.tm_cg_solve(op, x, pack(tl, L, eta, 0), n,
+                   tl.cg_params(1e-10, 500, tl.CG_MIXED, inner_prec=tl.F64, delta=0.1, check_every=1))
+    got = unpack(tl, L, x, 0, n)
+    assert np.abs(got[..., 2] * 2.0 ** 1000 * 2.0 ** 30 - got[..., 0]).max() <= 1e-8 * np.abs(got[..., 0]).max()
+    op.close()
