@@ -136,7 +136,6 @@ struct CgScalars {
   double delta2;
   double n12;     // 12 V complex components per field
   int max_iter;
-  int nrhs;
   int mixed;
 };
 
@@ -473,7 +472,6 @@ tm_status_t CgRun::setup() {
   sc.delta2 = mixed ? prm.delta * prm.delta : 0.0;
   sc.n12 = 12.0 * (double)g.Vh * npar;
   sc.max_iter = prm.max_iter;
-  sc.nrhs = nrhs;
   sc.mixed = mixed ? 1 : 0;
   // reductions over the parities the vectors live on
   part0 = partial + (schur ? nwarp : 0);

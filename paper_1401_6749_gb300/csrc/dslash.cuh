@@ -373,8 +373,8 @@ __device__ __forceinline__ void link_mv2(Cx<R> (&w)[6], const Mat3<R>& U, const 
       r0 = O::fma(-u.im, h0[b].im, r0); i0 = O::fma(u.im, h0[b].re, i0);
       r1 = O::fma(-u.im, h1[b].im, r1); i1 = O::fma(u.im, h1[b].re, i1);
     }
-    w[a] = {O::norm(r0), O::norm(i0)};
-    w[3 + a] = {O::norm(r1), O::norm(i1)};
+    w[a] = {r0, i0};
+    w[3 + a] = {r1, i1};
   }
 }
 
@@ -417,7 +417,7 @@ __device__ __forceinline__ void combine_dir(Cx<R> (&acc)[12], const Cx<R> (&wf)[
   Cx<R> d[6];
 #pragma unroll
   for (int k = 0; k < 6; ++k)
-    d[k] = {O::norm(O::fma(two, wf[k].re, -sum[k].re)), O::norm(O::fma(two, wf[k].im, -sum[k].im))};
+    d[k] = {O::fma(two, wf[k].re, -sum[k].re), O::fma(two, wf[k].im, -sum[k].im)};
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     acc[c] = add_ph<0>(acc[c], sum[c]);
@@ -466,13 +466,11 @@ __device__ __forceinline__ double warp_sum(double v) {
 // blocks (72 registers) is fastest for FP16/BF16 (8 blocks = 64 registers
 // spills), 6 for FP32.  Several systems per thread need registers in
 // proportion (4 blocks for 2, 2 for 4), so that the autotuner compares them
-// without forced spills.  FP64 and float-float are arithmetic bound and keep
-// their registers.  TM_DSLASH_MINBLOCKS (TM_DSLASH_MINBLOCKS_F32 for FP32
+// without forced spills.  FP64 is arithmetic bound and keeps its registers.  TM_DSLASH_MINBLOCKS (TM_DSLASH_MINBLOCKS_F32 for FP32
 // only) overrides the one-system value at build time.
 template <class S, int NR = 1>
 constexpr int dslash_min_blocks() {
   if constexpr (std::is_same<S, double>::value) return 1;
-  else if constexpr (std::is_same<S, FFloat>::value) return 2;
   else if constexpr (NR >= 4) return 2;
   else if constexpr (NR == 2) return 4;
 #ifdef TM_DSLASH_MINBLOCKS_F32
@@ -533,16 +531,12 @@ __device__ __forceinline__ double dslash_epilogue(const DslashArgs& a, const Epi
 #pragma unroll
     for (int q = 0; q < 12; ++q) out[q] = {O::mul(shop, acc[q].re), O::mul(shop, acc[q].im)};
   }
-  if constexpr (std::is_same<R, FF>::value) {
-#pragma unroll
-    for (int q = 0; q < 12; ++q) out[q] = {O::norm(out[q].re), O::norm(out[q].im)};
-  }
   if (a.c.out_inv) {  // A^-1 v = (v - i nu g5 v) / (1 + nu^2)
 #pragma unroll
     for (int q = 0; q < 12; ++q) {
       const R tw = q < 6 ? nu : -nu;
       const Cx<R> v = out[q];
-      out[q] = {O::mul(inv, O::norm(O::fma(tw, v.im, v.re))), O::mul(inv, O::norm(O::fma(-tw, v.re, v.im)))};
+      out[q] = {O::mul(inv, O::fma(tw, v.im, v.re)), O::mul(inv, O::fma(-tw, v.re, v.im))};
     }
   }
   double part = 0.0;
@@ -620,7 +614,7 @@ __global__ void __launch_bounds__(128, (dslash_min_blocks<S, NR>())) dslash_kern
     // forward hops use (1 - g) for M and (1 + g) for M^dag; backward the opposite
     constexpr int SF = DAG ? +1 : -1;
     constexpr int SB = -SF;
-// FP32/FP64/float-float: both hops of a direction combined (combine_dir), the
+// FP32/FP64: both hops of a direction combined (combine_dir), the
 // time-boundary sign on the projected spinor.  FP16/BF16: one hop at a time,
 // which holds fewer registers and spills less in this register-capped,
 // issue-bound kernel (measured faster); with 18-real links entirely on the
@@ -887,11 +881,18 @@ tm_status_t launch_nr(const tm_op* op, const DslashCall& c, cudaStream_t st) {
       const bool form = EPI == EPI_OUT || !c.custom || (c.centre == 2 && !c.out_inv);
       if (op->links_fx && form) return launch_one<S, RECON, DAG, EPI, 1, false, false, true>(op, c, st);
     }
-    if constexpr (std::is_same<S, FFloat>::value && EPI != EPI_CGUPD)
-      return launch_one<S, RECON, DAG, EPI, 1, false, false, true>(op, c, st);
-    // FP64 with links out of the fixed point's range: arithmetic-bound, one
-    // system per thread
-    return launch_one<S, RECON, DAG, EPI, 1>(op, c, st);
+    if constexpr (std::is_same<S, FFloat>::value) {
+      if constexpr (EPI == EPI_CGUPD) {  // float-float is no precision of an iteration
+        set_error("dslash: no CG update in float-float");
+        return TM_ERR_UNSUPPORTED;
+      } else {
+        return launch_one<S, RECON, DAG, EPI, 1, false, false, true>(op, c, st);
+      }
+    } else {
+      // FP64 on links that the fixed point does not take: arithmetic-bound, one
+      // system per thread
+      return launch_one<S, RECON, DAG, EPI, 1>(op, c, st);
+    }
   } else {
     if constexpr (kRawLinks<S, RECON>) {
       if (dslash_mma_on()) return launch_one<S, RECON, DAG, EPI, 1, false, true>(op, c, st);
