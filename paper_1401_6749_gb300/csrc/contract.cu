@@ -137,25 +137,81 @@ __global__ void mom_phase_kernel(Geom g, MomList mom, int q0, int nq, Cx<R>* ph)
 // m_ab(x) = sum_c conj(L_ac) R_bc formed once per site.  Per tile of 128 sites
 // each thread forms one site's m and the block loads the tile's phases into
 // shared memory; then warp w takes the sites w, w + 4, ..., lane (qg, cg) the
-// momenta qg QT .. qg QT + QT - 1 and the bilinears 2 cg, 2 cg + 1.  FP32 sums run
-// over eight sites and are then added with compensation (two-sum), so their
-// error stays that of a short sum.  Bound by the FMA pipe (64 FMAs per site and
+// momenta qg QT .. qg QT + QT - 1 and the bilinears 2 cg, 2 cg + 1.  Sums run over
+// eight sites and are then added (MomSum).  Bound by the FMA pipe (64 FMAs per site and
 // momentum); a pass per momentum, which it replaces, formed the 16 bilinears
 // and the phase again for each.  QT = 0: one momentum; the lane groups take its
 // terms of eight sites in turn and these are added in the order of the other
 // forms, so that a momentum's bits do not depend on the list it is asked in.
 constexpr int kMomTile = 128;
-__device__ __forceinline__ FF shfl_from(FF v, int l) {
-  return {__shfl_sync(0xffffffffu, v.hi, l), __shfl_sync(0xffffffffu, v.lo, l)};
-}
-template <class R>
-__device__ __forceinline__ R shfl_from(R v, int l) { return __shfl_sync(0xffffffffu, v, l); }
+
+// Sums of eight sites' terms (fma) and of such sums (add), by arithmetic type.
+//   FP32: plain, then compensated (two-sum).
+//   FP64: two chains of four sites, then plain.
+//   Float-float: as ff_fma, with the low parts' sums compensated, in the bilinears
+//   too.  Uncompensated, the sums over sites err as much as the bilinears: 5.4e-15 at
+//   zero momentum and 6.6e-15 at others (8^3 x 16); now 3.0e-15 and 3.5e-15 (a kernel
+//   per momentum, without sums over eight sites in float-float: 3.3e-15 and 3.6e-15).
+//   24^3 x 48, 12 systems, 19 momenta: 9.4 -> 11.8 ms.
+template <class R> struct MomSum;
+template <> struct MomSum<float> {
+  float s, e;
+  __device__ __forceinline__ void zero() { s = e = 0.0f; }
+  __device__ __forceinline__ void fma(int, float a, float b) { s = __fmaf_rn(a, b, s); }
+  __device__ __forceinline__ void end() {}
+  __device__ __forceinline__ void add(const MomSum& v) {
+    const FF f = ff_two_sum(s, v.s);
+    s = f.hi;
+    e = __fadd_rn(e, f.lo);
+  }
+  __device__ __forceinline__ MomSum from(int l) const { return {__shfl_sync(0xffffffffu, s, l), 0.0f}; }
+  __device__ __forceinline__ float term() const { return s; }  // of a single chain
+  __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+};
+template <> struct MomSum<double> {
+  double s, e;
+  __device__ __forceinline__ void zero() { s = e = 0.0; }
+  __device__ __forceinline__ void fma(int k, double a, double b) {
+    if (k < 4) s = __fma_rn(a, b, s);
+    else e = __fma_rn(a, b, e);
+  }
+  __device__ __forceinline__ void end() { s = __dadd_rn(s, e); }
+  __device__ __forceinline__ void add(const MomSum& v) { s = __dadd_rn(s, v.s); }
+  __device__ __forceinline__ MomSum from(int l) const { return {__shfl_sync(0xffffffffu, s, l), 0.0}; }
+  __device__ __forceinline__ double term() const { return s; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <> struct MomSum<FF> {
+  float s, lo, e;
+  __device__ __forceinline__ void zero() { s = lo = e = 0.0f; }
+  __device__ __forceinline__ void fma(int, FF a, FF b) {  // as ff_fma, with the rounding of the low part kept
+    const float p = __fmul_rn(a.hi, b.hi);
+    float q = __fmaf_rn(a.hi, b.hi, -p);
+    q = __fmaf_rn(a.hi, b.lo, q);
+    q = __fmaf_rn(a.lo, b.hi, q);
+    const FF f = ff_two_sum(s, p), g = ff_two_sum(lo, __fadd_rn(f.lo, q));
+    s = f.hi;
+    lo = g.hi;
+    e = __fadd_rn(e, g.lo);
+  }
+  __device__ __forceinline__ void end() {}
+  __device__ __forceinline__ void add(const MomSum& v) {
+    const FF f = ff_two_sum(s, v.s), g = ff_two_sum(lo, v.lo), h = ff_two_sum(g.hi, f.lo);
+    s = f.hi;
+    lo = h.hi;
+    e = __fadd_rn(e, __fadd_rn(v.e, __fadd_rn(g.lo, h.lo)));
+  }
+  __device__ __forceinline__ MomSum from(int l) const {
+    return {__shfl_sync(0xffffffffu, s, l), __shfl_sync(0xffffffffu, lo, l), __shfl_sync(0xffffffffu, e, l)};
+  }
+  __device__ __forceinline__ FF term() const { return ff_norm(FF{s, __fadd_rn(lo, e)}); }
+  __device__ __forceinline__ double value() const { return (double)s + ((double)lo + (double)e); }
+};
 template <class S, int QT>
 __global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const void* Lf, const void* Rf, int nsite,
                                                                int nchunk, const void* phases, MomList mom, int q0,
                                                                double* partial) {
   using R = typename Prec<S>::R;
-  using O = Ar<R>;
   extern __shared__ __align__(16) unsigned char mom_smem[];
   Cx<R>* sm = reinterpret_cast<Cx<R>*>(mom_smem);  // [site][8 pairs, swizzled by site][2]
   Cx<R>* sp = sm + kMomTile * 16;                  // [site][nq]
@@ -167,9 +223,9 @@ __global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const voi
   const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
   const int cg = lane & 7, qg = lane >> 3;
   const Cx<R>* ph = static_cast<const Cx<R>*>(phases) + (size_t)((t + par) & 1) * g.V3h * nq;
-  Cx<R> acc[NA][2], err[NA][2];
+  MomSum<R> acc[NA][2][2];  // [momentum][bilinear][re, im]
 #pragma unroll
-  for (int j = 0; j < NA; ++j) acc[j][0] = acc[j][1] = err[j][0] = err[j][1] = {(R)0, (R)0};
+  for (int j = 0; j < 4 * NA; ++j) acc[j >> 2][(j >> 1) & 1][j & 1].zero();
   const int iend = min(g.V3h, (chunk + 1) * nsite);
 #pragma unroll 1
   for (int i0 = chunk * nsite; i0 < iend; i0 += kMomTile) {
@@ -186,16 +242,18 @@ __global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const voi
       for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-          R zr = (R)0, zi = (R)0;
+          MomSum<R> zr, zi;
+          zr.zero();
+          zi.zero();
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
             const Cx<R> x = l[3 * a + c], y = r[3 * b + c];
-            zr = O::fma(x.re, y.re, zr);
-            zr = O::fma(x.im, y.im, zr);
-            zi = O::fma(x.re, y.im, zi);
-            zi = O::fma(-x.im, y.re, zi);
+            zr.fma(0, x.re, y.re);
+            zr.fma(0, x.im, y.im);
+            zi.fma(0, x.re, y.im);
+            zi.fma(0, -x.im, y.re);
           }
-          m[4 * a + b] = {O::norm(zr), O::norm(zi)};
+          m[4 * a + b] = {zr.term(), zi.term()};
         }
     }
     __syncthreads();  // the previous tile has been read
@@ -215,9 +273,9 @@ __global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const voi
     // one momentum: each lane group takes 32 sites of the warp's, and all add them in order
 #pragma unroll 1
     for (int s0 = ONE ? wq + 32 * qg : wq; s0 < (ONE ? wq + 32 * qg + 1 : rows); s0 += 32) {
-      Cx<R> z[NA][2];
+      MomSum<R> z[NA][2][2];
 #pragma unroll
-      for (int j = 0; j < NA; ++j) z[j][0] = z[j][1] = {(R)0, (R)0};
+      for (int j = 0; j < 4 * NA; ++j) z[j >> 2][(j >> 1) & 1][j & 1].zero();
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const int s = s0 + 4 * k;
@@ -226,31 +284,27 @@ __global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const voi
 #pragma unroll
           for (int j = 0; j < NA; ++j) {
             const Cx<R> p = sp[s * nq + (ONE ? 0 : qg * QT + j)];
-            z[j][0] = {O::fma(-p.im, m0.im, O::fma(p.re, m0.re, z[j][0].re)), O::fma(p.im, m0.re, O::fma(p.re, m0.im, z[j][0].im))};
-            z[j][1] = {O::fma(-p.im, m1.im, O::fma(p.re, m1.re, z[j][1].re)), O::fma(p.im, m1.re, O::fma(p.re, m1.im, z[j][1].im))};
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+              const Cx<R> m = c ? m1 : m0;
+              z[j][c][0].fma(k, p.re, m.re);
+              z[j][c][0].fma(k, -p.im, m.im);
+              z[j][c][1].fma(k, p.re, m.im);
+              z[j][c][1].fma(k, p.im, m.re);
+            }
           }
         }
       }
-      auto add = [](R& s, R& e, R v) {
-        if constexpr (std::is_same<R, float>::value) {
-          const FF f = ff_two_sum(s, v);
-          s = f.hi;
-          e = __fadd_rn(e, f.lo);
-        } else {
-          s = O::add(s, O::norm(v));
-        }
-      };
+#pragma unroll
+      for (int j = 0; j < 4 * NA; ++j) z[j >> 2][(j >> 1) & 1][j & 1].end();
 #pragma unroll
       for (int g0 = 0; g0 < (ONE ? 4 : 1); ++g0) {
         if (ONE && wq + 32 * g0 >= rows) break;
-        auto from = [&](R v) { return ONE ? shfl_from(v, 8 * g0 + cg) : v; };
 #pragma unroll
-        for (int j = 0; j < NA; ++j)
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            add(acc[j][c].re, err[j][c].re, from(z[j][c].re));
-            add(acc[j][c].im, err[j][c].im, from(z[j][c].im));
-          }
+        for (int j = 0; j < 4 * NA; ++j) {
+          const MomSum<R>& v = z[j >> 2][(j >> 1) & 1][j & 1];
+          acc[j >> 2][(j >> 1) & 1][j & 1].add(ONE ? v.from(8 * g0 + cg) : v);
+        }
       }
     }
   }
@@ -264,8 +318,8 @@ __global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const voi
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         double* w = red + ((size_t)wq * nq + qg * QT + j) * 32 + 2 * (2 * cg + c);
-        w[0] = (double)acc[j][c].re + (double)err[j][c].re;
-        w[1] = (double)acc[j][c].im + (double)err[j][c].im;
+        w[0] = acc[j][c][0].value();
+        w[1] = acc[j][c][1].value();
       }
   }
   __syncthreads();
@@ -280,10 +334,13 @@ __global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const voi
   }
 }
 
-// at most 32 momenta per pass: QT momenta per lane group, 0 for a single one.  4 and 6 are
+// momenta per pass: QT per lane group, 0 for a single one.  4 and 6 are
 // left out to keep the code small (a form is five kernels): they would save
 // lists of 13 to 16 and of 21 to 24 momenta a fifth and a seventh of the FMAs.
-constexpr int kMomPass = 32;
+// Float-float passes take 20: beyond, the sums (twelve registers per momentum of
+// a lane, twice) exceed the register file (24^3 x 48, 12 systems, 27 momenta: 23.2 ms
+// in one pass).
+static int mom_pass(tm_prec_t prec) { return prec == TM_PREC_FF ? 20 : 32; }
 static int mom_nq(int qt) { return qt == 0 ? 1 : 4 * qt; }
 static int mom_qt(int nq) {
   if (nq == 1) return 0;
@@ -896,7 +953,8 @@ extern "C" tm_status_t loop_contract_local_mom(const tm_geom_t* gg, const void* 
   const int nsite = mom_sites(g), nchunk = (g.V3h + nsite - 1) / nsite;
   // the table of phases of one pass behind the partial sums
   const size_t part = sizeof(double) * 32 * (size_t)n2 * g.L[3] * 2 * nchunk, cplx = prec == TM_PREC_F64 || prec == TM_PREC_FF ? 16 : 8;
-  const int nq_max = mom_nq(mom_qt(n_mom < kMomPass ? n_mom : kMomPass));
+  const int pass = mom_pass(prec);
+  const int nq_max = mom_nq(mom_qt(n_mom < pass ? n_mom : pass));
   double* scratch = nullptr;
   tm_status_t st = scratch_alloc((void**)&scratch, part + 2 * (size_t)g.V3h * nq_max * cplx, s);
   if (st != TM_OK) return st;
@@ -907,23 +965,29 @@ extern "C" tm_status_t loop_contract_local_mom(const tm_geom_t* gg, const void* 
     // per pass both fields once, and the table of phases written and read
     double tables = 0.0;
     int passes = 0;
-    for (int q0 = 0; q0 < n_mom; q0 += kMomPass, ++passes) {
-      const int nq = mom_nq(mom_qt(n_mom - q0 < kMomPass ? n_mom - q0 : kMomPass));
+    for (int q0 = 0; q0 < n_mom; q0 += pass, ++passes) {
+      const int nq = mom_nq(mom_qt(n_mom - q0 < pass ? n_mom - q0 : pass));
       if (mom_table(g, nrhs, nq)) tables += 2.0 * 2.0 * g.V3h * nq * (double)cplx;
     }
     TraceScope tr(s, prec_name(kNames, prec), passes * 2.0 * 24.0 * prec_size(prec) * 2.0 * g.Vh, tables, nrhs);
     st = by_prec_c(prec, [&](auto tag) {
       using S = decltype(tag);
-      for (int q0 = 0; q0 < n_mom; q0 += kMomPass) {
+      for (int q0 = 0; q0 < n_mom; q0 += pass) {
         tm_status_t ps;
-        switch (mom_qt(n_mom - q0 < kMomPass ? n_mom - q0 : kMomPass)) {
+        switch (mom_qt(n_mom - q0 < pass ? n_mom - q0 : pass)) {
           case 0: ps = mom_launch<S, 0>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
           case 1: ps = mom_launch<S, 1>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
           case 2: ps = mom_launch<S, 2>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
           case 3: ps = mom_launch<S, 3>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
           case 5: ps = mom_launch<S, 5>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
-          case 7: ps = mom_launch<S, 7>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
-          default: ps = mom_launch<S, 8>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
+          default:
+            if constexpr (std::is_same<S, FFloat>::value) {
+              ps = TM_ERR_UNSUPPORTED;  // not reached: mom_pass
+            } else if (n_mom - q0 <= 28) {
+              ps = mom_launch<S, 7>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s);
+            } else {
+              ps = mom_launch<S, 8>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s);
+            }
         }
         if (ps != TM_OK) return ps;
       }
