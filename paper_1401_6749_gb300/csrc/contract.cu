@@ -13,6 +13,7 @@
 // butterfly (transpose-reduce) leaves lane j with component j, the eight warp
 // results are added in order, and a final kernel adds the chunk partials in
 // order.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <limits>
@@ -119,14 +120,15 @@ struct MomList {
 };
 
 // The phases exp(-i p.x) of the sites of one slice, for both checkerboards of
-// (t + parity): [parity][i][nq] complex numbers, momenta q0 .. q0 + nq - 1 (zero
+// (t + parity): [group of nq momenta from q0 on][parity][i][nq] complex numbers (zero
 // beyond the list).
 template <class R>
-__global__ void mom_phase_kernel(Geom g, MomList mom, int q0, int nq, Cx<R>* ph) {
+__global__ void mom_phase_kernel(Geom g, MomList mom, int q0, int nq, int groups, Cx<R>* ph) {
   const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= 2L * g.V3h * nq) return;
-  const int q = q0 + (int)(k % nq);
-  const long pi = k / nq;
+  const long per = 2L * g.V3h * nq;
+  if (k >= per * groups) return;
+  const int q = q0 + (int)(k / per) * nq + (int)(k % nq);
+  const long pi = k % per / nq;
   Cx<R> v = {(R)0, (R)0};
   if (q < mom.n) v = mom_phase<R>(g, mom.q[q], site_of(g, (int)(pi / g.V3h), (int)(pi % g.V3h)));
   ph[k] = v;
@@ -207,7 +209,8 @@ template <> struct MomSum<FF> {
   __device__ __forceinline__ FF term() const { return ff_norm(FF{s, __fadd_rn(lo, e)}); }
   __device__ __forceinline__ double value() const { return (double)s + ((double)lo + (double)e); }
 };
-template <class S, int QT>
+// GROUPS: grid z holds [group of nq momenta][system]
+template <class S, int QT, bool GROUPS>
 __global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const void* Lf, const void* Rf, int nsite,
                                                                int nchunk, const void* phases, MomList mom, int q0,
                                                                double* partial) {
@@ -219,10 +222,16 @@ __global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const voi
   constexpr int nq = ONE ? 1 : 4 * QT, NA = ONE ? 1 : QT;  // momenta of the pass and of a lane
   const int chunk = (int)blockIdx.x;
   const int t = blockIdx.y >> 1, par = blockIdx.y & 1;
-  const int rhs = blockIdx.z;
+  int rhs = blockIdx.z;
   const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
   const int cg = lane & 7, qg = lane >> 3;
   const Cx<R>* ph = static_cast<const Cx<R>*>(phases) + (size_t)((t + par) & 1) * g.V3h * nq;
+  if constexpr (GROUPS) {
+    const int nrhs = gridDim.z / ((mom.n + nq - 1) / nq), grp = rhs / nrhs;
+    rhs -= grp * nrhs;
+    q0 = grp * nq;
+    ph += (size_t)grp * 2 * g.V3h * nq;
+  }
   MomSum<R> acc[NA][2][2];  // [momentum][bilinear][re, im]
 #pragma unroll
   for (int j = 0; j < 4 * NA; ++j) acc[j >> 2][(j >> 1) & 1][j & 1].zero();
@@ -267,7 +276,7 @@ __global__ void __launch_bounds__(kMomTile) mom_partial_kernel(Geom g, const voi
 #pragma unroll 1
       for (int q = 0; q < nq && q0 + q < mom.n; ++q) sp[threadIdx.x * nq + q] = mom_phase<R>(g, mom.q[q0 + q], st);
 #pragma unroll 1
-      for (int q = max(0, mom.n - q0); q < nq; ++q) sp[threadIdx.x * nq + q] = {(R)0, (R)0};
+      for (int q = mom.n - q0; q < nq; ++q) sp[threadIdx.x * nq + q] = {(R)0, (R)0};
     }
     __syncthreads();
     // one momentum: each lane group takes 32 sites of the warp's, and all add them in order
@@ -363,29 +372,41 @@ static int mom_sites(const Geom& g) {
 // 25.4 against 26.0 and 27.6; slower from 2^17 phases on (16^3 x 32, one momentum, float-float, one
 // system: 57 against 47; 4 systems, FP32: 54 against 42).
 static bool mom_table(const Geom& g, int nrhs, int nq) { return nq > 4 || 2.0 * g.Vh * nrhs * nq > 65536.0; }
+// Groups of at most eight momenta side by side in one launch, where the blocks of one
+// group leave SMs without one: as many as give every SM two blocks (1: no groups).
+// 8^3 x 16, one system, float-float, 4 and 19 momenta: 25 and 45 us against 32 and 77;
+// 16^3 x 32, 256 blocks, would take 102 and 302 us against 72 and 249.
+static int mom_groups(const Geom& g, int nrhs, int nchunk, int n, int* nq) {
+  const long k = 304 / (2L * g.L[3] * nchunk * nrhs);
+  if (k < 2 || n < 2) return 1;
+  const int most = (int)std::min<long>(std::max<long>(k, (n + 7) / 8), n);
+  *nq = mom_nq(mom_qt((n + most - 1) / most));
+  return (n + *nq - 1) / *nq;
+}
 
-template <class S, int QT>
+template <class S, int QT, bool GROUPS = false>
 static tm_status_t mom_launch(const Geom& g, const void* left, const void* right, int nrhs, const MomList& ml, int q0,
                               void* phases, int nsite, double* scratch, cudaStream_t s) {
   using R = typename Prec<S>::R;
   constexpr int nq = QT == 0 ? 1 : 4 * QT, smem = (int)sizeof(Cx<R>) * kMomTile * (16 + nq);
   if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(mom_partial_kernel<S, QT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+      cudaFuncSetAttribute(mom_partial_kernel<S, QT, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
           cudaSuccess) {
     set_error("loop_contract_local_mom: %s", cudaGetErrorString(cudaGetLastError()));
     return TM_ERR_CUDA;
   }
-  if (mom_table(g, nrhs, nq)) {
-    const long np = 2L * g.V3h * nq;
-    mom_phase_kernel<R><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(g, ml, q0, nq, static_cast<Cx<R>*>(phases));
+  const int groups = GROUPS ? (ml.n + nq - 1) / nq : 1;
+  if (mom_table(g, nrhs * groups, nq)) {
+    const long np = 2L * g.V3h * nq * groups;
+    mom_phase_kernel<R><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(g, ml, q0, nq, groups, static_cast<Cx<R>*>(phases));
     count_launch();
     TM_TRY(check_launch("loop_contract_local_mom phases"));
   } else {
     phases = nullptr;
   }
   const int nchunk = (g.V3h + nsite - 1) / nsite;
-  const dim3 grid(nchunk, 2 * g.L[3], nrhs);
-  mom_partial_kernel<S, QT><<<grid, kMomTile, smem, s>>>(g, left, right, nsite, nchunk, phases, ml, q0, scratch);
+  const dim3 grid(nchunk, 2 * g.L[3], nrhs * groups);
+  mom_partial_kernel<S, QT, GROUPS><<<grid, kMomTile, smem, s>>>(g, left, right, nsite, nchunk, phases, ml, q0, scratch);
   count_launch();
   return check_launch("loop_contract_local_mom");
 }
@@ -951,30 +972,37 @@ extern "C" tm_status_t loop_contract_local_mom(const tm_geom_t* gg, const void* 
     }
   const int n2 = nrhs * n_mom;
   const int nsite = mom_sites(g), nchunk = (g.V3h + nsite - 1) / nsite;
-  // the table of phases of one pass behind the partial sums
-  const size_t part = sizeof(double) * 32 * (size_t)n2 * g.L[3] * 2 * nchunk, cplx = prec == TM_PREC_F64 || prec == TM_PREC_FF ? 16 : 8;
+  // the table of phases of one launch behind the partial sums: of a pass, or of all groups
   const int pass = mom_pass(prec);
-  const int nq_max = mom_nq(mom_qt(n_mom < pass ? n_mom : pass));
+  int nq = mom_nq(mom_qt(std::min(n_mom, pass)));
+  const int groups = mom_groups(g, nrhs, nchunk, n_mom, &nq);
+  const size_t part = sizeof(double) * 32 * (size_t)n2 * g.L[3] * 2 * nchunk;
+  const size_t cplx = prec == TM_PREC_F64 || prec == TM_PREC_FF ? 16 : 8;
   double* scratch = nullptr;
-  tm_status_t st = scratch_alloc((void**)&scratch, part + 2 * (size_t)g.V3h * nq_max * cplx, s);
+  tm_status_t st = scratch_alloc((void**)&scratch, part + 2 * (size_t)g.V3h * nq * groups * cplx, s);
   if (st != TM_OK) return st;
   void* phases = reinterpret_cast<char*>(scratch) + part;
   {
     static const char* const kNames[kNumPrec] = {"localmom.f64", "localmom.f32", "localmom.f16", "localmom.bf16",
                                                   "localmom.ff"};
-    // per pass both fields once, and the table of phases written and read
+    // per pass or group both fields once, and the table of phases written and read
+    const int reads = groups > 1 ? groups : (n_mom + pass - 1) / pass;
     double tables = 0.0;
-    int passes = 0;
-    for (int q0 = 0; q0 < n_mom; q0 += pass, ++passes) {
-      const int nq = mom_nq(mom_qt(n_mom - q0 < pass ? n_mom - q0 : pass));
-      if (mom_table(g, nrhs, nq)) tables += 2.0 * 2.0 * g.V3h * nq * (double)cplx;
+    for (int r = 0; r < reads; ++r) {
+      const int q = groups > 1 ? nq : mom_nq(mom_qt(std::min(n_mom - r * pass, pass)));
+      if (mom_table(g, nrhs * groups, q)) tables += 2.0 * 2.0 * g.V3h * q * (double)cplx;
     }
-    TraceScope tr(s, prec_name(kNames, prec), passes * 2.0 * 24.0 * prec_size(prec) * 2.0 * g.Vh, tables, nrhs);
+    TraceScope tr(s, prec_name(kNames, prec), reads * 2.0 * 24.0 * prec_size(prec) * 2.0 * g.Vh, tables, nrhs);
     st = by_prec_c(prec, [&](auto tag) {
       using S = decltype(tag);
+      if (groups > 1) {
+        if (nq == 1) return mom_launch<S, 0, true>(g, left, right, nrhs, ml, 0, phases, nsite, scratch, s);
+        if (nq == 4) return mom_launch<S, 1, true>(g, left, right, nrhs, ml, 0, phases, nsite, scratch, s);
+        return mom_launch<S, 2, true>(g, left, right, nrhs, ml, 0, phases, nsite, scratch, s);
+      }
       for (int q0 = 0; q0 < n_mom; q0 += pass) {
         tm_status_t ps;
-        switch (mom_qt(n_mom - q0 < pass ? n_mom - q0 : pass)) {
+        switch (mom_qt(std::min(n_mom - q0, pass))) {
           case 0: ps = mom_launch<S, 0>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
           case 1: ps = mom_launch<S, 1>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;
           case 2: ps = mom_launch<S, 2>(g, left, right, nrhs, ml, q0, phases, nsite, scratch, s); break;

@@ -41,8 +41,9 @@ def _check(L, n, nmom, prec, mode, mom=None):
 
 
 @pytest.mark.parametrize("nmom", [1, 4, 5, 8, 12, 13, 20, 21, 28, 29, 32, 33, 64])
-def test_momentum_groups(nmom):
-    _check((6, 4, 8, 4), 2, nmom, "f32", "vv")
+@pytest.mark.parametrize("L", [(6, 4, 8, 4), (4, 4, 4, 40)])  # groups side by side (few blocks), and one after the other
+def test_momentum_groups(nmom, L):
+    _check(L, 2, nmom, "f32", "vv")
 
 
 @pytest.mark.parametrize("L", [(2, 2, 2, 2), (8, 8, 4, 2), (10, 6, 10, 4), (16, 12, 12, 2), (16, 16, 10, 4)])
@@ -54,6 +55,7 @@ def test_site_tiles(L, prec):
 @pytest.mark.parametrize("prec", ["ff", "f64"])
 def test_wide_full_pass(prec):
     _check((6, 4, 8, 4), 1, 32, prec, "gen")
+    _check((4, 4, 4, 40), 2, 32, prec, "gen")
 
 
 @pytest.mark.parametrize("p", [(0, 0, 0), (3, -1, 2)])
@@ -63,7 +65,7 @@ def test_single_momentum(p, prec):
 
 
 @pytest.mark.parametrize("prec", ["f16", "f32", "ff", "f64"])
-@pytest.mark.parametrize("L", [(8, 6, 4, 6), (16, 12, 12, 2), (10, 10, 14, 2)])
+@pytest.mark.parametrize("L", [(8, 6, 4, 6), (16, 12, 12, 2), (10, 10, 14, 2), (4, 4, 4, 40)])
 def test_list_independence(L, prec):
     """A momentum alone and in a list: the same bits."""
     tl = require_gpu()
@@ -87,7 +89,7 @@ def test_trace_bytes(nmom):
     """The record charges both fields once per pass of at most 32 momenta, and a
     small part more for the phases; not once per momentum."""
     tl = require_gpu()
-    L, n = (8, 8, 8, 16), 3
+    L, n = (16, 16, 16, 32), 3  # enough blocks for one group
     fields = 2 * n * 24 * 4 * int(np.prod(L))
     fl, fr = (pack(tl, L, synth.random_spinor(L, n, s), tl.F32) for s in (4, 5))
     out = torch.empty((n, nmom, 16, L[3], 2), dtype=torch.float64, device="cuda")
