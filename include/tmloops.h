@@ -371,7 +371,8 @@ tm_status_t loop_contract_oneD_il(tm_op_t *op, const void *left_il, const void *
  *   out[r][q][g][t] = sum_{x_t = t} exp(-i p_q . x) L_r(x)^dag (P Gamma_g) R_r(x),
  *   p_q = 2 pi (n_x / X, n_y / Y, n_z / Z),  mom = host array [n_mom][3] of (n_x, n_y, n_z)
  * (the paper computes zero-momentum loops; 1 <= n_mom <= 64, nrhs * n_mom <= 65535).
- * out: device [nrhs][n_mom][16][T][2].                                      */
+ * out: device [nrhs][n_mom][16][T][2].  The bits of a momentum depend neither on
+ * the list it is asked in nor on the other systems.                         */
 tm_status_t loop_contract_local_mom(const tm_geom_t *g, const void *left, const void *right,
                                     tm_prec_t prec, int nrhs, tm_loop_mode_t mode,
                                     const int *mom, int n_mom, double *out, tm_stream_t s);
